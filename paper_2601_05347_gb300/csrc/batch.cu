@@ -48,6 +48,7 @@ struct psi_batch {
   int64_t *d_qoff = nullptr;
   uint64_t *qk0 = nullptr, *qk1 = nullptr;
   uint32_t *qv0 = nullptr, *qv1 = nullptr;
+  uint32_t *d_nhard = nullptr;  // queries the k-NN's first kernel leaves to the second
   cudaStream_t last_stream = nullptr;
 };
 
@@ -495,7 +496,7 @@ static void batch_free(psi_batch *b) {
   for (void *p : {(void *)b->d_off, (void *)b->d_block_off, (void *)b->d_node_off, (void *)b->d_order,
                   (void *)b->d_root, (void *)b->d_queue, (void *)b->d_status, (void *)b->kA, (void *)b->kB,
                   (void *)b->vA, (void *)b->vB, (void *)b->d_qroot, (void *)b->d_qseg, (void *)b->d_qoff,
-                  (void *)b->qk0, (void *)b->qk1, (void *)b->qv0, (void *)b->qv1})
+                  (void *)b->qk0, (void *)b->qk1, (void *)b->qv0, (void *)b->qv1, (void *)b->d_nhard})
     DevMem::free(p, s);
   delete b;
 }
@@ -591,6 +592,7 @@ psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int
     if ((st = DevMem::alloc((void **)&b->d_root, sizeof(int32_t) * nidx, s))) break;
     if ((st = DevMem::alloc((void **)&b->d_queue, sizeof(uint32_t), s))) break;
     if ((st = DevMem::alloc((void **)&b->d_status, sizeof(int), s))) break;
+    if ((st = DevMem::alloc((void **)&b->d_nhard, sizeof(uint32_t), s))) break;
     if ((st = DevMem::alloc((void **)&b->kA, sizeof(uint64_t) * N, s))) break;
     if ((st = DevMem::alloc((void **)&b->kB, sizeof(uint64_t) * N, s))) break;
     if ((st = DevMem::alloc((void **)&b->vA, sizeof(uint32_t) * N, s))) break;
@@ -750,7 +752,12 @@ static psi_status batch_knn(psi_batch *b, const int32_t *d_q, const int64_t *d_q
   seed.phi = b->phi;
   seed.pkey = b->pool.pkey;
   seed.pos = reinterpret_cast<uint32_t *>(r.keys == b->qk0 ? b->qk1 : b->qk0);  // the sort's free key buffer
-  return run_knn_roots(tv, d_q, nq, k, r.vals, b->d_qroot, b->D, d_ids, d_d2, b->d_status, d_stats, s, seed);
+  KnnHard hard;
+  hard.q = seed.pos + nq;  // the other half of that buffer, and the sort's free position buffer
+  hard.pos = r.vals == b->qv0 ? b->qv1 : b->qv0;
+  hard.n = b->d_nhard;
+  return run_knn_roots(tv, d_q, nq, k, r.vals, b->d_qroot, b->D, d_ids, d_d2, b->d_status, d_stats, s, seed, -1, false,
+                       hard);
 }
 
 psi_status psi_batch_knn(psi_batch *b, const int32_t *d_q, const int64_t *d_qoffsets, int64_t nq, int32_t k,

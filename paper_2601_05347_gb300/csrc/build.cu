@@ -43,7 +43,8 @@ void free_nodes(NodeArrays &a, cudaStream_t s) {
 
 psi_status alloc_pool(Pool &p, int D, int64_t slots, cudaStream_t s) {
   p.cap_slots = slots;
-  const size_t c = (size_t)std::max<int64_t>(slots, 1);
+  // a multiple of four slots: the k-NN scan reads four at a time
+  const size_t c = (size_t)(ceil_div(std::max<int64_t>(slots, 1), 4) * 4);
   psi_status st;
   for (int d = 0; d < D; ++d)
     if ((st = DevMem::alloc((void **)&p.px[d], sizeof(int32_t) * c, s))) return st;

@@ -155,6 +155,13 @@ struct KnnSeed {
   const int32_t *leaf_node = nullptr;
 };
 
+// Scratch of the queries that the one-query-per-thread k-NN leaves to the
+// warp-per-query kernels (all null: that form is not used): nq entries each in
+// q and pos, and one counter.
+struct KnnHard {
+  uint32_t *q = nullptr, *pos = nullptr, *n = nullptr;
+};
+
 // k-NN of nq queries, each starting at qroot[q] (or tv.root when qroot is
 // null), in the given query order; d_stats (or null) receives traversal counts;
 // leaf_limit >= 0 says the leaves are exactly the nodes [0, leaf_limit);
@@ -164,5 +171,5 @@ struct KnnSeed {
 psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k, const uint32_t *order,
                          const int32_t *qroot, int D, uint32_t *out_id, int64_t *out_d2, int *status,
                          unsigned long long *d_stats, cudaStream_t s, const KnnSeed &seed,
-                         int64_t leaf_limit = -1, bool porth = false);
+                         int64_t leaf_limit = -1, bool porth = false, const KnnHard &hard = KnnHard());
 }  // namespace psi

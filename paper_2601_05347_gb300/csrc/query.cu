@@ -24,6 +24,7 @@
 #include "index.cuh"
 #include "keys.cuh"
 #include "klist.cuh"
+#include "knn.cuh"
 
 namespace psi {
 
@@ -34,7 +35,8 @@ struct QueryOrder {
   const uint32_t *order = nullptr;
   const uint64_t *keys = nullptr;
   int key_shift = 0;
-  uint32_t *spare = nullptr;  // nq free words (the key buffer the sort left unused)
+  uint32_t *spare = nullptr;    // 2 nq free words (the key buffer the sort left unused)
+  uint32_t *spare_v = nullptr;  // nq free words (the position buffer it left unused)
 };
 
 namespace {
@@ -42,26 +44,6 @@ namespace {
 constexpr int QW = 4;         // warps per block
 constexpr int STACK = 256;    // stack entries per warp (>= depth * fanout)
 constexpr uint32_t INSIDE = 0x80000000u;
-
-// Pruning key of a child box: the float bits of a lower bound of its squared
-// distance to the query, computed on the FP32 pipe (the ALU pipe is the
-// k-NN kernel's bottleneck): each gap is an exact int32 difference converted,
-// squared and summed with rounding toward -inf, so the bound never exceeds the
-// exact distance; a float at or below the exact k-th distance is at or below
-// that distance rounded to nearest, so comparing float bits never prunes a box
-// that holds a neighbour.
-template <int D>
-__device__ __forceinline__ uint32_t box_key_of(const int32_t *lo, const int32_t *hi, const int32_t *qc) {
-  float s = 0.0f;
-#pragma unroll
-  for (int d = 0; d < D; ++d) {
-    const int32_t q = qc[d];
-    const int32_t g = q < lo[d] ? lo[d] - q : (q > hi[d] ? q - hi[d] : 0);
-    const float gf = __int2float_rd(g);
-    s = __fadd_rd(s, __fmul_rd(gf, gf));
-  }
-  return __float_as_uint(s);
-}
 
 template <int D>
 __device__ __forceinline__ uint32_t box_key(const TreeView &t, uint32_t node, const int32_t *qc) {
@@ -86,20 +68,6 @@ __device__ __forceinline__ int box_relation(const TreeView &t, uint32_t node, co
   }
   return disjoint ? 0 : (inside ? 2 : 1);
 }
-
-struct KnnArgs {
-  TreeView t;
-  const int32_t *q;
-  int64_t nq;
-  int k;
-  const uint32_t *order;
-  const int32_t *qroot;  // per-query root (many indexes in one node array), or null
-  KnnSeed seed;        // SPaC: leaves scanned before the search
-  int64_t leaf_limit;  // >= 0: the leaves are exactly the nodes [0, leaf_limit) (one SPaC index)
-  uint32_t *out_id;
-  int64_t *out_d2;
-  int *status;
-};
 
 // Scan one leaf: every point whose (d2, id) beats the current k-th enters the
 // list (klist_offer: in bulk when many enter at once, the seed leaves of a
@@ -140,28 +108,12 @@ __device__ __forceinline__ void knn_scan_leaf(const TreeView &t, uint32_t node, 
   knn_scan_slots<D, KPL, EMPTY>(t, t.ref[node], t.cnt[node], qc, kl, k);
 }
 
-// 32-bit image of a non-negative distance for pruning: the float bits of the
-// distance rounded up, built from its two 32-bit halves (a conversion from a
-// 64-bit integer would run on the FP64 unit, which is very slow on this GPU).
-// A child key is its box distance rounded down, so a child whose key exceeds
-// the image of the k-th distance is farther than that distance: pruning by
-// keys never skips a node that could hold a neighbour; it may keep a few that
-// cannot, which costs time, not exactness.
-__device__ __forceinline__ uint32_t order_key(int64_t md) {
-  const uint32_t hi = (uint32_t)((uint64_t)md >> 32), lo = (uint32_t)md;
-  return __float_as_uint(__fmaf_ru(__uint2float_ru(hi), 4294967296.0f, __uint2float_ru(lo)));
-}
-
 struct KnnStats {
   // [0] internal nodes expanded, [1] leaves scanned, [2] points scanned, [3] queries,
   // [4] child descriptors read (children evaluated by the expansions)
   unsigned long long *c;
 };
 
-// Per-warp depth-first stack of the k-NN search: an expanded node pushes at
-// most F - 1 more entries than it pops, so depth x 31 + 32 entries suffice
-// (SPaC: 7 levels at 1e9 points; P-Orth: at most 2^D children per level).
-constexpr int KSTACK = 256;
 // Queries per warp of the grouped k-NN kernel (k <= 32, queries in curve order).
 constexpr int kGroup = 2;
 // Flag of a stack entry that is a leaf to scan (in its count word).
@@ -218,15 +170,16 @@ __global__ void k_knn_seed(const KnnSeed sd, const uint32_t *ref, const uint32_t
 // starts (so the order of the later pops matters little), and the search then
 // skips the seed leaves.  Seed (P-Orth): the leaf whose cell holds the query's
 // key (or the last leaf before it in key order), alone.
-template <int D, int KPL, bool STATS, bool BATCH>
+template <int D, int KPL, bool STATS, bool BATCH, bool LIST = false>
 __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
   // internal nodes still to visit: (node, key, first child, children)
   __shared__ uint4 s_stk[QW][KSTACK];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int64_t nw = (int64_t)gridDim.x * QW;
+  const int64_t nq = LIST ? (int64_t)*a.d_nq : a.nq;
   const TreeView &t = a.t;
   unsigned long long n_int = 0, n_leaf = 0, n_pts = 0, n_kids = 0;
-  for (int64_t qi = (int64_t)blockIdx.x * QW + w; qi < a.nq; qi += nw) {
+  for (int64_t qi = (int64_t)blockIdx.x * QW + w; qi < nq; qi += nw) {
     const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
     int32_t qc[D];
 #pragma unroll
@@ -528,7 +481,7 @@ __device__ __forceinline__ void knn_scan_group(const TreeView &t, uint32_t s0, i
 // same as k_knn's: exact (distance, id) order, each query pruned by its own
 // k-th distance.  Seeds: the distinct seed leaves of the group's queries are
 // scanned first, for all of them.
-template <int D, int G, bool STATS, bool RECHECK>
+template <int D, int G, bool STATS, bool RECHECK, bool LIST = false>
 __global__ __launch_bounds__(QW * 32) void k_knn_group(KnnArgs a, KnnStats stats) {
   static_assert(G <= 2 || !RECHECK, "a stack entry holds the box keys of two queries");
   // internal nodes still to visit: (first child, children) and, with RECHECK,
@@ -538,11 +491,12 @@ __global__ __launch_bounds__(QW * 32) void k_knn_group(KnnArgs a, KnnStats stats
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const TreeView &t = a.t;
   const KnnSeed &sd = a.seed;
-  const int64_t ngroups = (a.nq + G - 1) / G;
+  const int64_t nq = LIST ? (int64_t)*a.d_nq : a.nq;
+  const int64_t ngroups = (nq + G - 1) / G;
   unsigned long long n_int = 0, n_leaf = 0, n_pts = 0, n_kids = 0;
   for (int64_t gi = (int64_t)blockIdx.x * QW + w; gi < ngroups; gi += (int64_t)gridDim.x * QW) {
     const int64_t qi0 = gi * G;
-    const int ng = (int)min((int64_t)G, a.nq - qi0);
+    const int ng = (int)min((int64_t)G, nq - qi0);
     int32_t qc[G][D];
     uint32_t seed[G];
 #pragma unroll
@@ -979,13 +933,30 @@ psi_status query_order(const psi_index *ix, const int32_t *q, int64_t nq, QueryO
   qo.keys = r.keys;
   qo.key_shift = e.key_shift;
   qo.spare = reinterpret_cast<uint32_t *>(r.keys == qo.k0.p ? qo.k1.p : qo.k0.p);
+  qo.spare_v = r.vals == qo.v0.p ? qo.v1.p : qo.v0.p;
   return PSI_OK;
+}
+
+// Fewest queries for which the one-query-per-thread kernel is the faster one:
+// it needs the chip full of queries (a wave is 8 blocks of 128 per SM), more
+// of them the longer the lists and, on P-Orth, the more nodes its shared walk
+// visits.  Measured on 1e7 points, whole call, warp per query / this kernel, in
+// us: 2D SPaC-H 10-NN 1.5e5 queries 390 / 351, 3e5 642 / 458, 1e6 1707 / 923;
+// 3D uniform SPaC-H 10-NN 1.5e5 546 / 523, 1e6 2520 / 1477; 3D P-Orth 10-NN
+// 3e5 1752 / 1686, 1e6 4553 / 3271, 16-NN 3e5 2278 / 2796.
+static int64_t lane_min_queries(int D, int k, bool porth) {
+  const int64_t wave = (int64_t)num_sms() * 1024;
+  if (k > kLaneMaxK || (porth && D == 3 && k > 10)) return INT64_MAX;
+  if (!porth) return k <= 5 ? wave : k <= 10 ? wave * 3 / 2 : D == 2 ? wave * 2 : wave * 3;
+  if (k == 1) return wave;
+  if (D == 2) return k <= 10 ? wave * 2 : wave * 4;
+  return k <= 5 ? wave * 5 / 2 : wave * 4;
 }
 
 psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k, const uint32_t *order,
                          const int32_t *qroot, int D, uint32_t *out_id, int64_t *out_d2, int *status,
                          unsigned long long *d_stats, cudaStream_t s, const KnnSeed &seed, int64_t leaf_limit,
-                         bool porth) {
+                         bool porth, const KnnHard &hard) {
   if (nq == 0) return PSI_OK;
   KnnArgs a{tv, q, nq, k, order, qroot, seed, leaf_limit, out_id, out_d2, status};
   KnnStats stats{d_stats};
@@ -996,6 +967,36 @@ psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k
     }
     const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(nq, 256), (int64_t)num_sms() * 16));
     PSI_LAUNCH(k_knn_seed, gs, 256, 0, s, seed, tv.ref, order, nq, seed.pos);
+  }
+  if (hard.q && !d_stats && nq >= lane_min_queries(D, k, porth)) {
+    PSI_CK(cudaMemsetAsync(hard.n, 0, sizeof(uint32_t), s));
+    LaneArgs l{a, hard.q, hard.pos, hard.n};
+    psi_status st = run_knn_lane(l, D, porth, s);
+    if (st) return st;
+    // the queries it left out, a warp for each (or for two)
+    a.order = hard.q;
+    a.seed.pos = hard.pos;
+    a.d_nq = hard.n;
+#define KNN_LIST(DD, PP)                                                                                            \
+  do {                                                                                                              \
+    if (qroot)                                                                                                      \
+      PSI_LAUNCH_NAMED("k_knn", (k_knn<DD, 1, false, PP, true>),                                                    \
+                       resident_query_grid(k_knn<DD, 1, false, PP, true>, nq), QW * 32, 0, s, a, stats);            \
+    else                                                                                                            \
+      PSI_LAUNCH_NAMED("k_knn", (k_knn_group<DD, kGroup, false, PP, true>),                                         \
+                       resident_query_grid(k_knn_group<DD, kGroup, false, PP, true>, ceil_div(nq, kGroup)), QW * 32, \
+                       0, s, a, stats);                                                                             \
+  } while (0)
+    if (D == 2) {
+      if (porth) KNN_LIST(2, true);
+      else KNN_LIST(2, false);
+    } else {
+      if (porth) KNN_LIST(3, true);
+      else KNN_LIST(3, false);
+    }
+#undef KNN_LIST
+    PSI_CK(cudaGetLastError());
+    return PSI_OK;
   }
   const int kpl = k <= 32 ? 1 : (k <= 64 ? 2 : 4);
   // k <= 32 over one tree with queries in curve order: kGroup queries per warp
@@ -1069,7 +1070,13 @@ psi_status run_knn(const psi_index *ix, const int32_t *q, int64_t nq, int k, uin
   psi_status st = query_order(ix, q, nq, qo, s);
   if (st) return st;
   KnnSeed seed;
+  KnnHard hard;
+  Buf<uint32_t> nhard;
   if (qo.keys) {
+    if ((st = nhard.alloc(1, s))) return st;
+    hard.q = qo.spare + nq;
+    hard.pos = qo.spare_v;
+    hard.n = nhard.p;
     seed.qkey = qo.keys;
     seed.L = ix->L;
     seed.key_shift = qo.key_shift;
@@ -1082,7 +1089,7 @@ psi_status run_knn(const psi_index *ix, const int32_t *q, int64_t nq, int k, uin
     }
   }
   return run_knn_roots(ix->view(), q, nq, k, qo.order, nullptr, ix->D, out_id, out_d2, ix->d_status, d_stats, s,
-                       seed, ix->cfg.kind == PSI_PORTH ? -1 : ix->L, ix->cfg.kind == PSI_PORTH);
+                       seed, ix->cfg.kind == PSI_PORTH ? -1 : ix->L, ix->cfg.kind == PSI_PORTH, hard);
 }
 
 psi_status run_range_count(const psi_index *ix, const int32_t *boxes, int64_t nq, int64_t *counts, cudaStream_t s) {
