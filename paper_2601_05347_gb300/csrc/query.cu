@@ -865,35 +865,225 @@ __global__ __launch_bounds__(QW * 32) void k_range(RangeArgs a) {
   }
 }
 
-// One block per query segment: ascending sort of its ids.
-__global__ __launch_bounds__(1024) void k_sort_segments(const int64_t *offsets, int64_t nq, uint32_t *ids) {
-  __shared__ uint32_t sv[4096];
-  for (int64_t q = blockIdx.x; q < nq; q += gridDim.x) {
-    const int64_t b = offsets[q], len = offsets[q + 1] - b;
-    if (len <= 1) continue;
-    if (len <= 4096) {
-      for (int64_t j = threadIdx.x; j < len; j += blockDim.x) sv[j] = ids[b + j];
+// ---- ascending sort of each query's ids ------------------------------------
+// Bitonic sort of T * E values held E per thread (value e of thread t at
+// position t * E + e) by a group of T threads: strides below E between a
+// thread's own registers, strides below 32 E by warp shuffles, the others
+// through shared memory ([E][T]; T > 32 only).
+template <int T, int E>
+__device__ __forceinline__ void seg_bitonic(uint32_t (&v)[E], uint32_t *sm) {
+  const int t = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  // strides from .. 1 between the thread's own values: stage k < E, whose runs
+  // alternate inside the thread, or (k >= E) an ascending merge
+  auto own = [&](int from, int k) {
+#pragma unroll
+    for (int j = E / 2; j > 0; j >>= 1)
+      if (j <= from) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+          if (!(e & j)) {
+            const bool asc = k >= E || (e & k) == 0;
+            const uint32_t a = min(v[e], v[e | j]), b = max(v[e], v[e | j]);
+            v[e] = asc ? a : b;
+            v[e | j] = asc ? b : a;
+          }
+      }
+  };
+  // From stage E on a run is a thread's or several threads': the threads of a
+  // descending one hold complements, so that every exchange ascends.
+  uint32_t flip = 0;
+  auto turn = [&](int k) {
+    const uint32_t f = (t * E & k) == 0 ? 0u : 0xFFFFFFFFu;
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] ^= flip ^ f;
+    flip = f;
+  };
+#pragma unroll
+  for (int k = 2; k < E; k <<= 1) own(k / 2, k);
+  if (E > 1) {
+    turn(E);
+    own(E / 2, E);
+  }
+#pragma unroll 1
+  for (int k = 2 * E; k <= T * E; k <<= 1) {
+    turn(k);
+    int j = k / 2;
+    if (T > 32) {
+#pragma unroll 1
+      for (; j >= 32 * E; j >>= 1) {
+        __syncthreads();
+#pragma unroll
+        for (int e = 0; e < E; ++e) sm[e * T + t] = v[e];
+        __syncthreads();
+        const int x = t ^ (j / E);
+        const bool low = (t & (j / E)) == 0;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const uint32_t o = sm[e * T + x];
+          v[e] = low ? min(v[e], o) : max(v[e], o);
+        }
+      }
+    }
+#pragma unroll 1
+    for (; j >= E; j >>= 1) {
+      const bool low = (t & (j / E)) == 0;
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const uint32_t o = __shfl_xor_sync(0xFFFFFFFFu, v[e], j / E);
+        v[e] = low ? min(v[e], o) : max(v[e], o);
+      }
+    }
+    own(E / 2, k);
+  }
+}
+
+// Sorts ids[0, len), len <= T * E.  The order of the values on the way in is
+// free, so they are read coalesced; they leave through shared memory, where
+// the group holds T * (E + 1) words.
+template <int T, int E>
+__device__ __forceinline__ void seg_sort(uint32_t *ids, int len, uint32_t *sm) {
+  const int t = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  uint32_t v[E];
+#pragma unroll
+  for (int e = 0; e < E; ++e) v[e] = e * T + t < len ? ids[e * T + t] : 0xFFFFFFFFu;
+  seg_bitonic<T, E>(v, sm);
+  auto sync = [] {
+    if (T == 32)
+      __syncwarp();
+    else
       __syncthreads();
-      bitonic_ascending(
-          len, [&](int64_t x, int64_t y) { return sv[x] < sv[y]; },
-          [&](int64_t x, int64_t y) {
-            const uint32_t tmp = sv[x];
-            sv[x] = sv[y];
-            sv[y] = tmp;
-          });
-      for (int64_t j = threadIdx.x; j < len; j += blockDim.x) ids[b + j] = sv[j];
-      __syncthreads();
-    } else {
-      uint32_t *v = ids + b;
-      bitonic_ascending(
-          len, [&](int64_t x, int64_t y) { return v[x] < v[y]; },
-          [&](int64_t x, int64_t y) {
-            const uint32_t tmp = v[x];
-            v[x] = v[y];
-            v[y] = tmp;
-          });
+  };
+  sync();
+  constexpr int S = E > 1 ? E + 1 : 1;  // a word of padding per thread: no bank conflicts
+#pragma unroll
+  for (int e = 0; e < E; ++e) sm[t * S + e] = v[e];
+  sync();
+#pragma unroll
+  for (int e = 0; e < E; ++e) {
+    const int p = e * T + t;
+    if (p < len) ids[p] = sm[p / E * S + p % E];
+  }
+  sync();
+}
+
+// The segments by length, each class sorted by a kernel of its own: a warp per
+// segment up to 1024 ids, then blocks of 64, 128 and 512 threads.  Many values
+// per thread keep most of the network in registers: at 1024 ids, 15 of its 55
+// stages are shuffles (whose rate bounds it) with 32 values per thread, 30
+// with 8.  The classes are listed first and every warp or block takes the next
+// segment of its list: taken in strides over all segments, some found twice as
+// many of their class as others (890 us against 740).  5e4 boxes of 1259 ids on
+// average (6.3e7 ids): 590 us, against 6.1 ms for one 1024-thread block per
+// segment with a network in shared memory and a barrier per stage; bound by
+// instruction issue (about 110 per id and 32 lanes).
+constexpr int kSegClasses = 4;
+constexpr int kSeg0 = 1024, kSeg1 = 2048, kSeg2 = 4096;  // largest of classes 0 to 2
+
+struct SegLists {
+  uint32_t *list;  // [kSegClasses][nq]
+  uint32_t *ctr;   // [kSegClasses] lengths of the lists, [kSegClasses] next to take
+  int64_t nq;
+};
+
+__global__ __launch_bounds__(256) void k_seg_classes(const int64_t *offsets, SegLists l) {
+  const int lane = threadIdx.x & 31;
+  const int64_t rounds = (l.nq + 31) / 32 * 32;
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < rounds; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t len = q < l.nq ? offsets[q + 1] - offsets[q] : 0;
+    const int c = len < 2 ? -1 : (len > kSeg0) + (len > kSeg1) + (len > kSeg2);
+#pragma unroll
+    for (int x = 0; x < kSegClasses; ++x) {
+      const uint32_t m = __ballot_sync(0xFFFFFFFFu, c == x);
+      if (!m) continue;
+      uint32_t base = 0;
+      if (lane == 0) base = atomicAdd(&l.ctr[x], (uint32_t)__popc(m));
+      base = __shfl_sync(0xFFFFFFFFu, base, 0);
+      if (c == x) l.list[x * l.nq + base + __popc(m & lanemask_lt())] = (uint32_t)q;
     }
   }
+}
+
+// Class 0: a warp per segment, E chosen so that at least half of the positions
+// hold ids.
+__global__ __launch_bounds__(128, 8) void k_sort_seg_warp(const int64_t *offsets, SegLists l, uint32_t *ids) {
+  __shared__ uint32_t sm[4][32 * 33];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t n = l.ctr[0];
+  for (;;) {
+    uint32_t x = 0;
+    if (lane == 0) x = atomicAdd(&l.ctr[kSegClasses], 1u);
+    x = __shfl_sync(0xFFFFFFFFu, x, 0);
+    if (x >= n) break;
+    const int64_t q = l.list[x], b = offsets[q];
+    const int len = (int)(offsets[q + 1] - b);
+    if (len <= 32)
+      seg_sort<32, 1>(ids + b, len, sm[w]);
+    else if (len <= 64)
+      seg_sort<32, 2>(ids + b, len, sm[w]);
+    else if (len <= 128)
+      seg_sort<32, 4>(ids + b, len, sm[w]);
+    else if (len <= 256)
+      seg_sort<32, 8>(ids + b, len, sm[w]);
+    else if (len <= 512)
+      seg_sort<32, 16>(ids + b, len, sm[w]);
+    else
+      seg_sort<32, 32>(ids + b, len, sm[w]);
+  }
+}
+
+// Class C: a block of T threads per segment, of up to 32 T ids; longer ones
+// (past the last class) in place in global memory.
+template <int T, int C>
+__global__ __launch_bounds__(T, 1024 / T) void k_sort_seg_block(const int64_t *offsets, SegLists l, uint32_t *ids) {
+  extern __shared__ uint32_t sm_seg[];  // T * 33
+  __shared__ uint32_t next;
+  const uint32_t n = l.ctr[C];
+  for (;;) {
+    if (threadIdx.x == 0) next = atomicAdd(&l.ctr[kSegClasses + C], 1u);
+    __syncthreads();
+    const uint32_t x = next;
+    __syncthreads();
+    if (x >= n) break;
+    const int64_t q = l.list[C * l.nq + x], b = offsets[q], len = offsets[q + 1] - b;
+    if (C == kSegClasses - 1 && len > 32 * T) {
+      uint32_t *v = ids + b;
+      bitonic_ascending(
+          len, [&](int64_t i, int64_t j) { return v[i] < v[j]; },
+          [&](int64_t i, int64_t j) {
+            const uint32_t tmp = v[i];
+            v[i] = v[j];
+            v[j] = tmp;
+          });
+    } else if (C == kSegClasses - 1 && len <= 16 * T) {
+      seg_sort<T, 16>(ids + b, (int)len, sm_seg);
+    } else {
+      seg_sort<T, 32>(ids + b, (int)len, sm_seg);
+    }
+  }
+}
+
+template <int T, int C>
+psi_status launch_sort_seg(const int64_t *offsets, const SegLists &l, uint32_t *ids, cudaStream_t s) {
+  const size_t smem = sizeof(uint32_t) * T * 33;
+  if (smem > 48 * 1024)
+    PSI_CK(cudaFuncSetAttribute(k_sort_seg_block<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PSI_LAUNCH_NAMED("k_sort_seg_block", (k_sort_seg_block<T, C>),
+                   (int)std::min<int64_t>(l.nq, (int64_t)num_sms() * (1024 / T)), T, smem, s, offsets, l, ids);
+  return PSI_OK;
+}
+
+psi_status sort_segments(const int64_t *offsets, int64_t nq, uint32_t *ids, cudaStream_t s) {
+  Buf<uint32_t> list, ctr;
+  psi_status st;
+  if ((st = list.alloc(kSegClasses * nq, s)) || (st = ctr.alloc(2 * kSegClasses, s))) return st;
+  PSI_CK(cudaMemsetAsync(ctr.p, 0, sizeof(uint32_t) * 2 * kSegClasses, s));
+  const SegLists l{list.p, ctr.p, nq};
+  PSI_LAUNCH(k_seg_classes, (int)std::min<int64_t>(ceil_div(nq, 256), (int64_t)num_sms() * 8), 256, 0, s, offsets, l);
+  PSI_LAUNCH(k_sort_seg_warp, (int)std::min<int64_t>(ceil_div(nq, 4), (int64_t)num_sms() * 8), 128, 0, s, offsets, l, ids);
+  if ((st = launch_sort_seg<64, 1>(offsets, l, ids, s)) || (st = launch_sort_seg<128, 2>(offsets, l, ids, s)) ||
+      (st = launch_sort_seg<512, 3>(offsets, l, ids, s)))
+    return st;
+  return PSI_OK;
 }
 
 // Grid of a grid-stride query kernel: the blocks that are resident at once
@@ -1113,8 +1303,10 @@ psi_status run_range_emit(const psi_index *ix, const int32_t *boxes, int64_t nq,
     PSI_LAUNCH_NAMED("k_range_emit", (k_range<2, true>), resident_query_grid(k_range<2, true>, nq), QW * 32, 0, s, a);
   else
     PSI_LAUNCH_NAMED("k_range_emit", (k_range<3, true>), resident_query_grid(k_range<3, true>, nq), QW * 32, 0, s, a);
-  if (sorted)
-    PSI_LAUNCH(k_sort_segments, (int)std::min<int64_t>(nq, (int64_t)num_sms() * 2), 1024, 0, s, offsets, nq, ids);
+  if (sorted) {
+    psi_status st = sort_segments(offsets, nq, ids, s);
+    if (st) return st;
+  }
   PSI_CK(cudaGetLastError());
   return PSI_OK;
 }
