@@ -153,6 +153,9 @@ struct KnnSeed {
   // P-Orth: node of each leaf of the key-ordered leaf list, whose cell base
   // keys sep_key then holds; null for SPaC, where leaf i is node i
   const int32_t *leaf_node = nullptr;
+  // self_bits > 0 (one SPaC index, few queries, qkey null): each query finds its
+  // own seed, from its key on the curve `curve` over self_bits bits per coordinate
+  int self_bits = 0, curve = 0;
 };
 
 // Scratch of the queries that the one-query-per-thread k-NN leaves to the

@@ -134,6 +134,22 @@ __device__ __forceinline__ int64_t seed_search(FirstKey first_key, int64_t n, ui
   return lo > 0 ? lo - 1 : 0;
 }
 
+// The same search by a whole warp (32 probes per step: four steps for 1e6
+// positions), for one query: its steps are dependent loads.
+__device__ __forceinline__ int64_t seed_search_warp(const uint64_t *first_key, int64_t n, uint64_t key) {
+  const int lane = threadIdx.x & 31;
+  int64_t lo = 0, hi = n;  // first position whose first key is greater
+  while (hi - lo > 32) {
+    const int64_t len = hi - lo;
+    const int c = __popc(__ballot_sync(0xFFFFFFFFu, first_key[lo + len * (lane + 1) / 33] <= key));
+    const int64_t l0 = lo;
+    if (c > 0) lo = l0 + len * c / 33 + 1;
+    if (c < 32) hi = l0 + len * (c + 1) / 33;
+  }
+  lo += __popc(__ballot_sync(0xFFFFFFFFu, lo + lane < hi && first_key[lo + lane] <= key));
+  return lo > 0 ? lo - 1 : 0;
+}
+
 // Seed position of every query (queries in curve order), one thread each:
 // SPaC, the node of the last leaf of the query's index whose first key is at
 // most the query's key; P-Orth, the position in the key-ordered leaf list of
@@ -170,7 +186,7 @@ __global__ void k_knn_seed(const KnnSeed sd, const uint32_t *ref, const uint32_t
 // starts (so the order of the later pops matters little), and the search then
 // skips the seed leaves.  Seed (P-Orth): the leaf whose cell holds the query's
 // key (or the last leaf before it in key order), alone.
-template <int D, int KPL, bool STATS, bool BATCH, bool LIST = false>
+template <int D, int KPL, bool STATS, bool BATCH, bool LIST = false, bool SELF = false, bool WIDE = false>
 __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
   // internal nodes still to visit: (node, key, first child, children)
   __shared__ uint4 s_stk[QW][KSTACK];
@@ -178,6 +194,11 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
   const int64_t nw = (int64_t)gridDim.x * QW;
   const int64_t nq = LIST ? (int64_t)*a.d_nq : a.nq;
   const TreeView &t = a.t;
+  __shared__ alignas(16) uint8_t s_tab[SELF ? kCurveTabBytes : 16];
+  if (SELF && a.seed.curve == CURVE_HILBERT) {
+    curve_table_init<D, CURVE_HILBERT>(s_tab);
+    __syncthreads();
+  }
   unsigned long long n_int = 0, n_leaf = 0, n_pts = 0, n_kids = 0;
   for (int64_t qi = (int64_t)blockIdx.x * QW + w; qi < nq; qi += nw) {
     const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
@@ -197,7 +218,13 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
       lb = sd.node_off[sg];
       L = (sd.off[sg + 1] - sd.off[sg] + sd.phi - 1) / sd.phi;
     }
-    if (sd.qkey && root >= 0) {
+    if (SELF) {
+      bool bad;  // (a query may lie outside the grid; its seed is then any leaf)
+      const uint64_t key = sd.curve == CURVE_HILBERT ? point_key<D, CURVE_HILBERT>(s_tab, qc, sd.self_bits, bad)
+                                                     : point_key<D, CURVE_MORTON>(s_tab, qc, sd.self_bits, bad);
+      s_lo = s_hi = seed_search_warp(sd.sep_key, sd.L, key);
+      knn_scan_leaf<D, KPL, true>(t, (uint32_t)s_lo, qc, kl, a.k);
+    } else if (sd.qkey && root >= 0) {
       const int64_t pos = sd.pos[qi];  // k_knn_seed
       if (L > 0) {
         // P-Orth: pos is a position in the key-ordered leaf list
@@ -244,20 +271,23 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
     // comes back here as `pl` (its lane 0 stands for the leaf).  Each lane
     // loads its child's reference and count with its box, so a popped entry
     // needs no further load before its own children are read.
+    // WIDE (P-Orth): each group of CW lanes has a node (or leaf entry) of its own.
+    constexpr int CW = WIDE ? 8 : 32;  // at least 2^D
+    const int cl = lane % CW;
     auto expand = [&](uint32_t c0, int nk, bool pl, uint32_t pkey) {
-      const uint32_t c = c0 + (uint32_t)lane;
+      const uint32_t c = c0 + (uint32_t)cl;
       uint32_t key = 0xFFFFFFFFu;  // above any k-th distance key
       bool leafc = false;
       uint32_t cref = 0;
       int ccnt = 0;
       if (pl) {
-        if (lane == 0) {
+        if (cl == 0) {
           key = pkey;
           leafc = true;
           cref = c0;
           ccnt = nk;
         }
-      } else if (lane < nk) {  // every node of every layout holds a point
+      } else if (cl < nk) {  // every node of every layout holds a point
         cref = t.ref[c];
         if (a.leaf_limit >= 0) {
           leafc = (int64_t)c < a.leaf_limit;
@@ -396,11 +426,21 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
         uint32_t c0 = t.ref[root], pkey = 0;
         int nk = t.kids[root];
         bool pl = false;
+        if (WIDE && lane >= CW) nk = 0;
         for (;;) {
           expand(c0, nk, pl, pkey);
           uint4 e = make_uint4(0, 0, 0, 0);
           bool more = false;
-          while (sp > 0) {
+          // WIDE: the top entries, one per group of lanes, while the stack has
+          // room for the most that single pops may add (2^D - 1 per level)
+          while (WIDE && sp > 0 && !more) {
+            const int g = lane / CW, take = sp <= 64 ? min(sp, 32 / CW) : 1;
+            e = g < take ? s_stk[w][sp - 1 - g] : make_uint4(0, 0xFFFFFFFFu, 0, 0);
+            sp -= take;
+            if (e.y > kdk) e = make_uint4(0, 0, 0, 0);  // no children
+            more = __any_sync(0xFFFFFFFFu, e.w != 0);
+          }
+          while (!WIDE && sp > 0) {
             e = s_stk[w][--sp];
             if (e.y <= kdk) {  // else farther than the k-th distance found since the push
               more = true;
@@ -1219,6 +1259,38 @@ psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k
     PSI_CK(cudaGetLastError());
     return PSI_OK;
   }
+  // few queries on a SPaC tree: each warp finds its query's seed leaf itself
+  // (its steps are dependent loads, a few microseconds; without the seed the
+  // search entered 2.6 to 7 times as many leaves: 1e3 10-NN on 1e7 Varden
+  // points, 2D SPaC-H 65 -> 36 us, 3D SPaC-Z 287 -> 35 us).  For k > 32 the
+  // search is long beside what the seed saves: 0.85 to 1.18 times as fast.  On
+  // P-Orth, whose nearest-box-first descent is near its floor, a seed of 32
+  // points around the query in key order cost more than it saved (41 -> 51 us).
+  if (seed.self_bits > 0 && kpl == 1 && !d_stats) {
+    if (D == 2)
+      PSI_LAUNCH_NAMED("k_knn", (k_knn<2, 1, false, false, false, true>),
+                       resident_query_grid(k_knn<2, 1, false, false, false, true>, nq), QW * 32, 0, s, a, stats);
+    else
+      PSI_LAUNCH_NAMED("k_knn", (k_knn<3, 1, false, false, false, true>),
+                       resident_query_grid(k_knn<3, 1, false, false, false, true>, nq), QW * 32, 0, s, a, stats);
+    PSI_CK(cudaGetLastError());
+    return PSI_OK;
+  }
+  // Few queries on P-Orth leave the chip waiting on the chain of dependent node
+  // loads of each search: up to four nodes are expanded at once, at the price of
+  // some that single steps would have pruned (1e3 10-NN on 1e6 3D uniform
+  // points 29.3 -> 25.5 us a call; queries away from 1e7 3D Varden points 123
+  // -> 104 us).
+  if (porth && kpl == 1 && !order && !d_stats) {
+    if (D == 2)
+      PSI_LAUNCH_NAMED("k_knn", (k_knn<2, 1, false, true, false, false, true>),
+                       resident_query_grid(k_knn<2, 1, false, true, false, false, true>, nq), QW * 32, 0, s, a, stats);
+    else
+      PSI_LAUNCH_NAMED("k_knn", (k_knn<3, 1, false, true, false, false, true>),
+                       resident_query_grid(k_knn<3, 1, false, true, false, false, true>, nq), QW * 32, 0, s, a, stats);
+    PSI_CK(cudaGetLastError());
+    return PSI_OK;
+  }
 #define KNN_CASE1(DD, KK, BB)                                                                          \
   do {                                                                                                 \
     if (d_stats)                                                                                       \
@@ -1277,6 +1349,12 @@ psi_status run_knn(const psi_index *ix, const int32_t *q, int64_t nq, int k, uin
       seed.sep_key = ix->pl.key;
       seed.leaf_node = ix->leaf_node;
     }
+  }
+  if (!qo.keys && ix->L > 0 && ix->cfg.kind != PSI_PORTH) {  // few queries, not sorted
+    seed.self_bits = ix->cfg.coord_bits;
+    seed.curve = ix->curve;
+    seed.sep_key = ix->sep_key;
+    seed.L = ix->L;
   }
   return run_knn_roots(ix->view(), q, nq, k, qo.order, nullptr, ix->D, out_id, out_d2, ix->d_status, d_stats, s,
                        seed, ix->cfg.kind == PSI_PORTH ? -1 : ix->L, ix->cfg.kind == PSI_PORTH, hard);
