@@ -591,18 +591,20 @@ struct FKnnArgs {
   uint32_t *out_id;
   double *out_d2;
   int *status;
+  const uint32_t *d_nq = nullptr;  // listed queries (order): their number, at most nq
 };
 
 // One warp per query: depth-first search entering the nearest unvisited child
 // first (the integer k-NN kernel's traversal, with float boxes and double
 // distances); the children of each level on the path are kept in shared memory.
-template <int D, int KPL>
+template <int D, int KPL, bool LIST = false>
 __global__ __launch_bounds__(FQW * 32) void k_fknn(FKnnArgs a) {
   __shared__ uint32_t s_key[FQW][FMAXLVL][32];
   __shared__ uint32_t s_c0[FQW][FMAXLVL], s_mask[FQW][FMAXLVL], s_leaf[FQW][FMAXLVL];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const FView &t = a.t;
-  for (int64_t qi = (int64_t)blockIdx.x * FQW + w; qi < a.nq; qi += (int64_t)gridDim.x * FQW) {
+  const int64_t nq = LIST ? (int64_t)*a.d_nq : a.nq;
+  for (int64_t qi = (int64_t)blockIdx.x * FQW + w; qi < nq; qi += (int64_t)gridDim.x * FQW) {
     const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
     float qc[D];
 #pragma unroll
@@ -697,6 +699,382 @@ __global__ __launch_bounds__(FQW * 32) void k_fknn(FKnnArgs a) {
         a.out_d2[q * a.k + e] = kl.d[r];
       }
     }
+  }
+}
+
+// ---- k-NN with one query per thread (k <= 16, many queries) --------------------
+// The method of knn_lane.cu on this tree: 32 neighbouring queries share one
+// depth-first walk, the (leaf, query) pairs it finds are scanned a lane each,
+// and each query keeps the K smallest float images of its distances and the
+// slots of the points within the bound they give; double distances are taken
+// only of those, at the end (FP64 runs at 1/64 of the FP32 rate here).
+//
+// Images are the bits of float distances rounded to nearest: at most D + 3
+// roundings of 2^-24 each away from the exact value, so two images in the wrong
+// order differ by less than kImageSlack units (denormal sums: an absolute
+// error of D units at most).
+//
+// A query's seeds are the 32 or more slots around the leaf it reaches by
+// entering the nearest child box at every level: slots follow the tree's
+// order, so they are its neighbours there.  Queries that are not finite, that
+// find more points within their bound than they can note, or whose search is
+// long are listed for k_fknn.
+constexpr int FLT = 128, FLW = FLT / 32;
+constexpr int kFPool = 128, kFStack = 96, kFSpare = 10, kFLong = 96;
+constexpr uint32_t kFMaxLeaf = 1024;  // slots of a pair; a longer leaf is a pile of duplicates
+constexpr uint32_t kImageSlack = 32;
+template <int K>
+constexpr int kFNotes = K + 22;
+
+struct FLaneArgs {
+  FKnnArgs a;
+  int64_t n;
+  uint32_t *hq, *hn;  // listed queries and their number (zero on entry)
+};
+
+template <int D>
+__device__ __forceinline__ uint32_t fimage(const float *const *px, const float *qc, uint32_t slot) {
+  float f = 0.0f;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    const float g = px[d][slot] - qc[d];
+    f = fmaf(g, g, f);
+  }
+  return __float_as_uint(f);
+}
+
+template <int D, int K>
+struct FLaneSearch {
+  const FView &t;
+  float qc[D];
+  uint32_t F[K];  // the K smallest images, ascending (a shorter list starts with zeros)
+  uint32_t kb;    // images above it cannot be among the k nearest
+  uint32_t *note;  // FLT apart
+  int nn, nd;
+  bool full;
+  static constexpr int kRoom = kFNotes<K> - kFSpare;
+
+  __device__ __forceinline__ void init(int k) {
+    nn = nd = 0;
+    full = false;
+    kb = 0xFFFFFFFEu;
+#pragma unroll
+    for (int j = 0; j < K; ++j) F[j] = j < K - k ? 0u : 0xFFFFFFFEu - kImageSlack;
+  }
+  __device__ __forceinline__ void take(uint32_t f) {
+#pragma unroll
+    for (int x = K - 1; x > 0; --x) F[x] = max(F[x - 1], min(F[x], f));
+    F[0] = min(F[0], f);
+  }
+  __device__ __forceinline__ void set_bound() { kb = F[K - 1] + kImageSlack; }
+  __device__ __forceinline__ void digest() {
+    const int most = __reduce_max_sync(0xFFFFFFFFu, nn - nd);
+    for (int j = 0; j < most; j += 2) {
+      uint32_t f[2];
+#pragma unroll
+      for (int u = 0; u < 2; ++u) {
+        f[u] = 0xFFFFFFFEu - kImageSlack;
+        if (nd + j + u < nn) f[u] = fimage<D>(t.px, qc, note[(nd + j + u) * FLT]);
+      }
+      take(f[0]);
+      take(f[1]);
+    }
+    nd = nn;
+    set_bound();
+  }
+  __device__ __forceinline__ void compact() {
+    const int most = __reduce_max_sync(0xFFFFFFFFu, nn);
+    int o = 0;
+    for (int j = 0; j < most; ++j)
+      if (j < nn) {
+        const uint32_t slot = note[j * FLT];
+        if (fimage<D>(t.px, qc, slot) <= kb) note[FLT * o++] = slot;
+      }
+    nn = nd = o;
+    if (o > kRoom) {
+      full = true;
+      nn = nd = 0;
+    }
+  }
+};
+
+template <int D, int K>
+__global__ __launch_bounds__(FLT, K <= 10 ? 7 : 6) void k_fknn_lane(FLaneArgs la) {
+  constexpr int CW = D <= 3 ? 8 : 1 << D;  // lanes per expanded node
+  __shared__ uint2 s_stk[FLW][kFStack];    // nodes to expand: (first child, children)
+  __shared__ uint32_t s_ref[FLW][kFPool], s_cnt[FLW][kFPool], s_key[FLW][kFPool];  // pairs waiting
+  __shared__ uint32_t s_note[kFNotes<K>][FLT];
+  __shared__ int s_nn[FLT];
+  const FKnnArgs &a = la.a;
+  const FView &t = a.t;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int64_t qi = (int64_t)blockIdx.x * FLT + tid;
+  const bool valid = qi < a.nq;
+  const uint32_t q = a.order[valid ? qi : a.nq - 1];
+  FLaneSearch<D, K> S{t};
+  S.note = &s_note[0][tid];
+  S.init(a.k);
+  bool hard = false;
+#pragma unroll
+  for (int d = 0; d < D; ++d) {
+    S.qc[d] = a.q[(int64_t)q * D + d];
+    hard |= !(fabsf(S.qc[d]) < __int_as_float(0x7F800000));
+  }
+  hard &= valid;
+  bool act = valid && !hard;
+  // the leaf reached through the nearest child boxes
+  uint32_t wlo = 0, whi = 0;  // the seeds' slots
+  if (act) {
+    uint32_t u = 0;
+    int nk = t.kids[0];
+    while (nk > 0) {
+      const uint32_t c0 = t.ref[u];
+      float best = __int_as_float(0x7F800000);
+      uint32_t bu = c0;
+      for (int c = 0; c < nk; ++c) {
+        const float f = fbox_lower<D>(t, c0 + (uint32_t)c, S.qc);
+        if (f < best) {
+          best = f;
+          bu = c0 + (uint32_t)c;
+        }
+      }
+      u = bu;
+      nk = t.kids[u];
+    }
+    const int64_t s0 = t.ref[u], e0 = s0 + t.cnt[u];
+    const int64_t more = max((int64_t)0, (32 - (e0 - s0) + 1) / 2);
+    wlo = (uint32_t)max((int64_t)0, s0 - more);
+    whi = (uint32_t)min(la.n, e0 + more);
+    if (whi - wlo > kFMaxLeaf) {
+      hard = true;
+      act = false;
+    } else {
+      for (uint32_t s = wlo; s < whi; ++s) S.take(fimage<D>(t.px, S.qc, s));
+      S.set_bound();
+    }
+  }
+  __syncwarp();
+  int np = 0, total = 0;
+  // the seeds' own slots first, then the tree
+  {
+    const uint32_t m = __ballot_sync(0xFFFFFFFFu, act);
+    if (act) {
+      const int p = __popc(m & lanemask_lt());
+      s_ref[w][p] = wlo;
+      s_cnt[w][p] = (whi - wlo) << 5 | (uint32_t)lane;
+      s_key[w][p] = 0;
+    }
+    np = __popc(m);
+  }
+  bool seeds = true, started = false;
+  uint32_t m = 0, lm = 0, gk = 0, c0 = 0;
+  int sp = 0, nk = 0;
+  bool leafc = false;
+  float lo_[D], hi_[D], glo[D], ghi[D];
+  uint32_t cref = 0;
+  int ccnt = 0;
+  for (;;) {
+    bool more = true;
+    if (!seeds) {
+      for (;;) {
+        if (!m) {
+          if (!started) {  // the root as the only child of a virtual node
+            started = true;
+            c0 = 0;
+            nk = lane == 0 ? 1 : 0;
+          } else if (sp == 0) {
+            more = false;
+            break;
+          } else {
+            const int g = lane / CW, take = min(sp, 32 / CW);
+            __syncwarp();
+            const uint2 e = g < take ? s_stk[w][sp - 1 - g] : make_uint2(0u, 0u);
+            __syncwarp();
+            sp -= take;
+            c0 = e.x - (uint32_t)(g * CW);
+            nk = (int)e.y - lane % CW;
+          }
+          const uint32_t c = c0 + (uint32_t)lane;
+          bool near = false;
+          leafc = false;
+          if (nk > 0) {
+            cref = t.ref[c];
+            const int ck = t.kids[c], cn = t.cnt[c];
+            leafc = ck == 0;
+            ccnt = leafc ? cn : ck;
+            float f = 0.0f;
+#pragma unroll
+            for (int d = 0; d < D; ++d) {
+              lo_[d] = t.lo[d][c];
+              hi_[d] = t.hi[d][c];
+              const float g = fmaxf(0.0f, fmaxf(__fsub_rd(lo_[d], ghi[d]), __fsub_rd(glo[d], hi_[d])));
+              f = __fadd_rd(f, __fmul_rd(g, g));
+            }
+            near = __float_as_uint(f) <= gk;
+          }
+          m = __ballot_sync(0xFFFFFFFFu, near);
+          lm = __ballot_sync(0xFFFFFFFFu, leafc);
+          continue;
+        }
+        const int src = __ffs(m) - 1;
+        m &= m - 1;
+        float f = 0.0f;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+          const float lo = __shfl_sync(0xFFFFFFFFu, lo_[d], src), hi = __shfl_sync(0xFFFFFFFFu, hi_[d], src);
+          const float g = fmaxf(0.0f, fmaxf(__fsub_rd(lo, S.qc[d]), __fsub_rd(S.qc[d], hi)));
+          f = __fadd_rd(f, __fmul_rd(g, g));
+        }
+        const uint32_t key = __float_as_uint(f);
+        const uint32_t bref = __shfl_sync(0xFFFFFFFFu, cref, src);
+        const int bcnt = __shfl_sync(0xFFFFFFFFu, ccnt, src);
+        bool need = act && key <= S.kb;
+        if ((lm >> src) & 1u) {
+          // the leaf's slots that are not among the seeds: the window holds a
+          // whole leaf, so it cuts another at one end only
+          uint32_t s0 = bref, s1 = bref + (uint32_t)bcnt;
+          if (s0 >= wlo && s0 < whi)
+            s0 = min(s1, whi);
+          else if (s0 < wlo && s1 > wlo)
+            s1 = wlo;
+          need &= s1 > s0;
+          if (bcnt > (int)kFMaxLeaf) {
+            hard |= need;
+            act &= !need;
+            continue;
+          }
+          const uint32_t nm = __ballot_sync(0xFFFFFFFFu, need);
+          if (need) {
+            const int p = np + __popc(nm & lanemask_lt());
+            s_ref[w][p] = s0;
+            s_cnt[w][p] = (s1 - s0) << 5 | (uint32_t)lane;
+            s_key[w][p] = key;
+            ++total;
+          }
+          np += __popc(nm);
+          if (np > kFPool - 32) break;
+        } else if (__any_sync(0xFFFFFFFFu, need)) {
+          if (sp < kFStack) {
+            if (lane == 0) s_stk[w][sp] = make_uint2(bref, (uint32_t)bcnt);
+            ++sp;
+          } else {  // too many nodes waiting
+            hard |= need;
+            act &= !need;
+          }
+        }
+      }
+    }
+    // the pool, a lane per pair
+    s_nn[tid] = S.nn;
+    __syncwarp();
+    for (int x0 = 0; x0 < np; x0 += 32) {
+      const bool has = x0 + lane < np;
+      const uint32_t e = has ? s_cnt[w][x0 + lane] : (uint32_t)lane;
+      const int o = (int)(e & 31u);  // the pair's query
+      float oq[D];
+#pragma unroll
+      for (int d = 0; d < D; ++d) oq[d] = __shfl_sync(0xFFFFFFFFu, S.qc[d], o);
+      const uint32_t okb = __shfl_sync(0xFFFFFFFFu, S.full ? 0u : S.kb, o);
+      const bool ofull = __shfl_sync(0xFFFFFFFFu, S.full, o);
+      uint32_t s = 0, s1 = 0;
+      if (has && !ofull && s_key[w][x0 + lane] <= okb) {
+        s = s_ref[w][x0 + lane];
+        s1 = s + (e >> 5);
+      }
+      int *on = &s_nn[w * 32 + o];
+      uint32_t *onote = &s_note[0][w * 32 + o];
+      for (; s < s1; ++s)
+        if (fimage<D>(t.px, oq, s) <= okb) {
+          const int p = atomicAdd(on, 1);
+          if (p < kFNotes<K>) onote[FLT * p] = s;
+        }
+      __syncwarp();
+      S.nn = s_nn[tid];
+      if (S.nn > kFNotes<K>) {  // some were not noted
+        S.full = true;
+        S.nn = S.nd = 0;
+      }
+      if (__any_sync(0xFFFFFFFFu, S.nn > FLaneSearch<D, K>::kRoom)) {
+        if (seeds)
+          S.nd = S.nn;
+        else
+          S.digest();
+        S.compact();
+      }
+      s_nn[tid] = S.nn;
+      __syncwarp();
+    }
+    np = 0;
+    if (!more) break;
+    if (seeds) {
+      S.nd = S.nn;
+      seeds = false;
+      hard |= act && (S.full || S.kb >= 0x7F800000u);  // too few points in the seeds
+      act &= !hard;
+      if (!__any_sync(0xFFFFFFFFu, act)) break;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {  // box around the active queries
+        const float inf = __int_as_float(0x7F800000);
+        float l = act ? S.qc[d] : inf, h = act ? S.qc[d] : -inf;
+#pragma unroll
+        for (int o = 16; o; o >>= 1) {
+          l = fminf(l, __shfl_xor_sync(0xFFFFFFFFu, l, o));
+          h = fmaxf(h, __shfl_xor_sync(0xFFFFFFFFu, h, o));
+        }
+        glo[d] = l;
+        ghi[d] = h;
+      }
+    } else {
+      S.digest();
+      if (S.full || total > kFLong) {
+        hard |= act;
+        act = false;
+      }
+    }
+    gk = __reduce_max_sync(0xFFFFFFFFu, act ? S.kb : 0u);
+  }
+
+  // the notes in exact (distance, id) order; the bits of non-negative doubles
+  // order as integers do
+  constexpr int N = K == 1 ? 4 : 16;
+  int64_t od[N];
+  uint32_t oi[N];
+#pragma unroll
+  for (int x = 0; x < N; ++x) {
+    od[x] = 0x7FF0000000000000ll;
+    oi[x] = 0xFFFFFFFFu;
+    if (x < S.nn) {
+      const uint32_t slot = S.note[x * FLT];
+      od[x] = __double_as_longlong(fpoint_d2<D>(S.qc, t.px, slot));
+      oi[x] = t.pid[slot];
+    }
+  }
+  pair_network(od, oi);
+  const int most = __reduce_max_sync(0xFFFFFFFFu, S.nn);
+  for (int x = N; x < most; ++x) {
+    int64_t d2 = 0x7FF0000000000000ll;
+    uint32_t id = 0xFFFFFFFFu;
+    if (x < S.nn) {
+      const uint32_t slot = S.note[x * FLT];
+      d2 = __double_as_longlong(fpoint_d2<D>(S.qc, t.px, slot));
+      id = t.pid[slot];
+    }
+    if (__any_sync(0xFFFFFFFFu, pair_less(d2, id, od[K - 1], oi[K - 1]))) pair_insert<K>(od, oi, d2, id);
+  }
+  hard |= valid && S.full;
+  const uint32_t hm = __ballot_sync(0xFFFFFFFFu, hard);
+  uint32_t hbase = 0;
+  if (hm && lane == 0) hbase = atomicAdd(la.hn, (uint32_t)__popc(hm));
+  hbase = __shfl_sync(0xFFFFFFFFu, hbase, 0);
+  if (hard) {
+    la.hq[hbase + __popc(hm & lanemask_lt())] = q;
+  } else if (valid) {
+#pragma unroll
+    for (int x = 0; x < K; ++x)
+      if (x < a.k) {
+        a.out_id[(int64_t)q * a.k + x] = oi[x];
+        a.out_d2[(int64_t)q * a.k + x] = __longlong_as_double(od[x]);
+      }
   }
 }
 
@@ -821,6 +1199,33 @@ psi_status forth_knn_d(const psi_forth *ix, const float *q, int64_t nq, int k, u
   }
   FKnnArgs a{fview(ix), q, nq, k, order, ids, d2, ix->d_status};
   const int g = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(nq, FQW), (int64_t)num_sms() * 16));
+  // One query per thread needs the chip full of queries (a wave is 8 blocks of
+  // 128 per SM); the wider the nodes, the longer its shared walk beside the
+  // other kernel's.  Whole call on 3e6 uniform points, warp / thread per query,
+  // in us: 3D 10-NN 5e4 queries 912 / 522, 1.5e5 2382 / 733, 1e6 14743 / 2108
+  // (away from clustered points 5e4 1909 / 2059, 1.5e5 5097 / 4462); 5D 10-NN
+  // 5e4 2112 / 3633, 1.5e5 5545 / 4642, 1e6 35167 / 11712.
+  const int64_t wave = (int64_t)num_sms() * 1024;
+  const int64_t lane_min = D <= 3 ? wave / 2 : D == 4 ? wave : wave * 3 / 2;
+  if (k <= 16 && order && nq >= lane_min && ix->N > 0) {
+    Buf<uint32_t> hn;
+    if ((st = hn.alloc(1, s))) return st;
+    PSI_CK(cudaMemsetAsync(hn.p, 0, sizeof(uint32_t), s));
+    // the buffer that the sort left unused holds the listed queries
+    FLaneArgs l{a, ix->n, order == v0.p ? v1.p : v0.p, hn.p};
+    const unsigned gl = (unsigned)ceil_div(nq, FLT);
+    if (k == 1)
+      PSI_LAUNCH_NAMED("k_fknn", (k_fknn_lane<D, 1>), gl, FLT, 0, s, l);
+    else if (k <= 10)
+      PSI_LAUNCH_NAMED("k_fknn", (k_fknn_lane<D, 10>), gl, FLT, 0, s, l);
+    else
+      PSI_LAUNCH_NAMED("k_fknn", (k_fknn_lane<D, 16>), gl, FLT, 0, s, l);
+    a.order = l.hq;
+    a.d_nq = l.hn;
+    PSI_LAUNCH_NAMED("k_fknn", (k_fknn<D, 1, true>), g, FQW * 32, 0, s, a);
+    PSI_CK(cudaGetLastError());
+    return PSI_OK;
+  }
   if (k <= 32)
     PSI_LAUNCH_NAMED("k_fknn", (k_fknn<D, 1>), g, FQW * 32, 0, s, a);
   else if (k <= 64)

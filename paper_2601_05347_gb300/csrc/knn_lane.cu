@@ -194,45 +194,6 @@ struct LaneSearch {
   }
 };
 
-// Orders two (distance, id) pairs.
-__device__ __forceinline__ void pair_order(int64_t &da, uint32_t &ia, int64_t &db, uint32_t &ib) {
-  const bool sw = pair_less(db, ib, da, ia);
-  const int64_t d = sw ? db : da, e = sw ? da : db;
-  const uint32_t i = sw ? ib : ia, j = sw ? ia : ib;
-  da = d;
-  db = e;
-  ia = i;
-  ib = j;
-}
-
-// Batcher's odd-even merge sort of N pairs in registers, from stage (P, Q) on.
-template <int N, int P = 1, int Q = 1>
-__device__ __forceinline__ void pair_network(int64_t (&d)[N], uint32_t (&i)[N]) {
-#pragma unroll
-  for (int x = 0; x + Q < N; ++x)
-    if (x >= Q % P && (x - Q % P) % (2 * Q) < Q && x / (2 * P) == (x + Q) / (2 * P))
-      pair_order(d[x], i[x], d[x + Q], i[x + Q]);
-  if constexpr (Q > 1)
-    pair_network<N, P, Q / 2>(d, i);
-  else if constexpr (2 * P < N)
-    pair_network<N, 2 * P, 2 * P>(d, i);
-}
-
-// Takes (cd, ci) into the first K of a sorted list; one above them changes nothing.
-template <int K, int N>
-__device__ __forceinline__ void pair_insert(int64_t (&d)[N], uint32_t (&i)[N], int64_t cd, uint32_t ci) {
-  bool p[K];
-#pragma unroll
-  for (int j = 0; j < K; ++j) p[j] = pair_less(cd, ci, d[j], i[j]);
-#pragma unroll
-  for (int j = K - 1; j > 0; --j) {
-    d[j] = p[j - 1] ? d[j - 1] : (p[j] ? cd : d[j]);
-    i[j] = p[j - 1] ? i[j - 1] : (p[j] ? ci : i[j]);
-  }
-  d[0] = p[0] ? cd : d[0];
-  i[0] = p[0] ? ci : i[0];
-}
-
 // Squared diagonal of a node's box, rounded down.
 template <int D>
 __device__ __forceinline__ float box_diag2(const TreeView &t, uint32_t node) {
