@@ -156,7 +156,9 @@ typedef struct psi_batch psi_batch;
  * SPAC_H).  `threads` is the thread-block size of the build (256, 512, 1024; 0
  * = 512); cfg->radix_bits is the digit width of the build's block sort (0 or 8:
  * 8-bit digits; 11: 11-bit digits, with 256 or 512 threads only).  The index
- * layout does not depend on either.  Allocates everything the build needs, so psi_batch_build and
+ * layout does not depend on either; with both 0, a batch whose points are mostly
+ * in a few large indexes is built by device-wide sorts instead of a block per
+ * index.  Allocates everything the build needs, so psi_batch_build and
  * psi_batch_knn allocate nothing and can be captured in a CUDA graph.
  * Synchronises `stream`. */
 psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int32_t nidx, int32_t threads,
@@ -164,7 +166,8 @@ psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int
 
 /* Builds every index of the batch (Algorithm 3 per index: curve keys, (key, id)
  * sort, leaf wrapping, summaries) in ONE persistent kernel launch: each thread
- * block takes whole indexes, largest first, from an atomic queue.  Each index
+ * block takes whole indexes, largest first, from an atomic queue (or, see
+ * psi_batch_create, in the launches of one sort of the whole batch).  Each index
  * gets exactly the layout psi_build would give it.  d_pts [total][dim] and
  * d_ids [total] are read during the call only. */
 psi_status psi_batch_build(psi_batch *b, const int32_t *d_pts, const uint32_t *d_ids, void *stream);

@@ -28,6 +28,8 @@ struct psi_batch {
   psi_config cfg;
   int D = 2, phi = 32, C = 64, F = 32, curve = 0, key_bits = 60, threads = 512;
   int rb = 8;  // digit width of the block sort
+  int seg_bits = 0;   // bits of an index number
+  bool wide = false;  // built by device-wide sorts (few large indexes) instead of a block each
   int nidx = 0;
   int64_t total = 0;
   std::vector<int64_t> off, leaves, node_off, block_off, nodes_per;
@@ -133,6 +135,62 @@ __device__ __forceinline__ void block_excl_scan_digits(const uint32_t (&v)[DPT],
     e[q] = run;
     run += v[q];
   }
+}
+
+// The F-ary summary levels over the L leaves at nodes [node0, node0 + L), bottom
+// up, by the whole block (a warp per parent); returns the root.
+template <int D>
+__device__ __forceinline__ int64_t batch_summary(const BuildArgs &a, int64_t node0, int64_t L) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  int64_t coff = 0, csize = L, total = L;
+  int level = 0;
+  while (csize > 1) {
+    const int64_t par = (csize + a.F - 1) / a.F;
+    ++level;
+    for (int64_t j = w; j < par; j += W) {
+      const int64_t c0 = j * a.F;
+      const int nk = (int)min((int64_t)a.F, csize - c0);
+      int32_t lo[D], hi[D];
+      int32_t cnt = 0;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        lo[d] = INT32_MAX;
+        hi[d] = INT32_MIN;
+      }
+      if (lane < nk) {
+        const int64_t c = node0 + coff + c0 + lane;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+          lo[d] = a.nodes.lo[d][c];
+          hi[d] = a.nodes.hi[d][c];
+        }
+        cnt = a.nodes.cnt[c];
+      }
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        lo[d] = __reduce_min_sync(0xFFFFFFFFu, lo[d]);
+        hi[d] = __reduce_max_sync(0xFFFFFFFFu, hi[d]);
+      }
+      cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
+      if (lane == 0) {
+        const int64_t pn = node0 + total + j;
+#pragma unroll
+        for (int d = 0; d < D; ++d) {
+          a.nodes.lo[d][pn] = lo[d];
+          a.nodes.hi[d][pn] = hi[d];
+        }
+        a.nodes.cnt[pn] = cnt;
+        a.nodes.ref[pn] = (uint32_t)(node0 + coff + c0);
+        a.nodes.kids[pn] = nk;
+        a.nodes.depth[pn] = level;
+      }
+    }
+    __syncthreads();
+    coff = total;
+    total += par;
+    csize = par;
+  }
+  return node0 + total - 1;
 }
 
 template <int D, int CURVE, int BT, int RB>
@@ -384,57 +442,225 @@ __global__ __launch_bounds__(BT) void k_batch_build(BuildArgs a) {
     }
     __syncthreads();
     // U: summary levels
-    int64_t coff = 0, csize = L, total = L;
-    int level = 0;
-    while (csize > 1) {
-      const int64_t par = (csize + a.F - 1) / a.F;
-      ++level;
-      for (int64_t j = w; j < par; j += W) {
-        const int64_t c0 = j * a.F;
-        const int nk = (int)min((int64_t)a.F, csize - c0);
-        int32_t lo[D], hi[D];
-        int32_t cnt = 0;
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-          lo[d] = INT32_MAX;
-          hi[d] = INT32_MIN;
-        }
-        if (lane < nk) {
-          const int64_t c = node0 + coff + c0 + lane;
-#pragma unroll
-          for (int d = 0; d < D; ++d) {
-            lo[d] = a.nodes.lo[d][c];
-            hi[d] = a.nodes.hi[d][c];
-          }
-          cnt = a.nodes.cnt[c];
-        }
-#pragma unroll
-        for (int d = 0; d < D; ++d) {
-          lo[d] = __reduce_min_sync(0xFFFFFFFFu, lo[d]);
-          hi[d] = __reduce_max_sync(0xFFFFFFFFu, hi[d]);
-        }
-        cnt = __reduce_add_sync(0xFFFFFFFFu, cnt);
-        if (lane == 0) {
-          const int64_t pn = node0 + total + j;
-#pragma unroll
-          for (int d = 0; d < D; ++d) {
-            a.nodes.lo[d][pn] = lo[d];
-            a.nodes.hi[d][pn] = hi[d];
-          }
-          a.nodes.cnt[pn] = cnt;
-          a.nodes.ref[pn] = (uint32_t)(node0 + coff + c0);
-          a.nodes.kids[pn] = nk;
-          a.nodes.depth[pn] = level;
-        }
-      }
-      __syncthreads();
-      coff = total;
-      total += par;
-      csize = par;
-    }
-    if (tid == 0) a.root[ix] = (int32_t)(node0 + total - 1);
+    const int64_t top = batch_summary<D>(a, node0, L);
+    if (tid == 0) a.root[ix] = (int32_t)top;
     __syncthreads();
   }
+}
+
+// ---- Device-wide build ---------------------------------------------------------
+// A block builds an index at about 18 ns per point, so a batch whose points
+// are mostly in a few large indexes leaves most SMs idle while their blocks
+// finish.  Such a batch is sorted as a whole: by the low 8 key bits first, then
+// by (index number, the other key bits) in one word, with the device's digit
+// passes; the leaves of all indexes are then gathered at once.  The layout is
+// the same.  256 indexes of 1e3 to 1e6 points (3.7e7 in all), build: 19.3 ms by
+// blocks, 5.0 ms device-wide; 4096 of them (5.95e8) take 67 ms by blocks.
+
+// Index that position p of the concatenated arrays belongs to.
+__device__ __forceinline__ int segment_of(const int64_t *off, int nidx, int64_t p) {
+  int lo = 0, hi = nidx;  // last segment with off <= p
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (off[mid] <= p)
+      lo = mid;
+    else
+      hi = mid;
+  }
+  return lo;
+}
+
+template <int D, int CURVE>
+__global__ __launch_bounds__(256) void k_wide_keys(const int32_t *pts, int64_t n, int bits, uint64_t *keys,
+                                                   uint32_t *vals, int *status) {
+  __shared__ alignas(16) uint8_t htab[kCurveTabBytes];
+  curve_table_init<D, CURVE>(htab);
+  __syncthreads();
+  const uint64_t mask = (uint64_t(1) << (D * bits)) - 1;  // (a coordinate out of range is reported; its key stays in range)
+  bool bad_any = false;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    int32_t c[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) c[d] = pts[i * D + d];
+    bool bad;
+    keys[i] = point_key<D, CURVE>(htab, c, bits, bad) & mask;
+    vals[i] = (uint32_t)i;
+    bad_any |= bad;
+  }
+  if (bad_any) atomicOr(status, ST_RANGE);
+}
+
+// key -> index number above the key without its low 8 bits.
+__global__ void k_wide_segment(const int64_t *off, int nidx, int shift, const uint32_t *vals, int64_t n,
+                               uint64_t *keys) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    keys[i] = (uint64_t)segment_of(off, nidx, vals[i]) << shift | keys[i] >> 8;
+}
+
+// The full key of every sorted position, from its point.
+template <int D, int CURVE>
+__global__ __launch_bounds__(256) void k_wide_full(const int32_t *pts, const uint32_t *vals, int64_t n, int bits,
+                                                   uint64_t *keys) {
+  __shared__ alignas(16) uint8_t htab[kCurveTabBytes];
+  curve_table_init<D, CURVE>(htab);
+  __syncthreads();
+  const uint64_t mask = (uint64_t(1) << (D * bits)) - 1;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t v = vals[i];
+    int32_t c[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) c[d] = pts[v * D + d];
+    bool bad;
+    keys[i] = point_key<D, CURVE>(htab, c, bits, bad) & mask;
+  }
+}
+
+// Runs of equal keys within an index, put in id order: up to 32 by a thread,
+// longer ones listed for k_wide_tie_long.  (A segment is looked up only where
+// two neighbouring keys are equal.)
+__global__ void k_wide_ties(const uint64_t *keys, uint32_t *vals, const uint32_t *ids, const int64_t *off, int nidx,
+                            int64_t n, int64_t *longs, uint32_t *n_long) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i + 1 < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const uint64_t k = keys[i];
+    if (keys[i + 1] != k) continue;
+    const int sg = segment_of(off, nidx, i);
+    const int64_t b = off[sg], e = off[sg + 1];
+    if (i + 1 >= e || (i > b && keys[i - 1] == k)) continue;
+    int64_t x = i + 2;
+    while (x < e && keys[x] == k && x - i <= 32) ++x;
+    if (x - i > 32) {
+      longs[atomicAdd(n_long, 1u)] = i;  // at most one per 33 positions
+      continue;
+    }
+    for (int64_t y = i + 1; y < x; ++y) {
+      const uint32_t v = vals[y], id = ids[v];
+      int64_t z = y - 1;
+      while (z >= i && ids[vals[z]] > id) {
+        vals[z + 1] = vals[z];
+        --z;
+      }
+      vals[z + 1] = v;
+    }
+  }
+}
+
+__global__ __launch_bounds__(1024) void k_wide_tie_long(const uint64_t *keys, uint32_t *vals, const uint32_t *ids,
+                                                        const int64_t *off, int nidx, const int64_t *longs,
+                                                        const uint32_t *n_long) {
+  for (int64_t r = blockIdx.x; r < (int64_t)*n_long; r += gridDim.x) {
+    const int64_t s = longs[r];
+    const uint64_t k = keys[s];
+    int64_t lo = s, hi = off[segment_of(off, nidx, s) + 1];  // first position past the run
+    while (lo < hi) {
+      const int64_t mid = (lo + hi) >> 1;
+      if (keys[mid] == k)
+        lo = mid + 1;
+      else
+        hi = mid;
+    }
+    uint32_t *v = vals + s;
+    bitonic_ascending(
+        lo - s, [&](int64_t x, int64_t y) { return ids[v[x]] < ids[v[y]]; },
+        [&](int64_t x, int64_t y) {
+          const uint32_t t = v[x];
+          v[x] = v[y];
+          v[y] = t;
+        });
+  }
+}
+
+// A warp per leaf of any index (leaf numbers run over all indexes, which
+// block_off delimits): its points into its block, its box, its node.
+template <int D>
+__global__ __launch_bounds__(256) void k_wide_gather(const uint64_t *keys, const uint32_t *vals, BuildArgs a,
+                                                     int64_t leaves) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t g = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; g < leaves; g += warps) {
+    int ix = segment_of(a.block_off, a.nidx, g);
+    const int64_t j = g - a.block_off[ix];
+    const int64_t b = a.off[ix] + j * a.phi;
+    const int cnt = (int)min((int64_t)a.phi, a.off[ix + 1] - b);
+    int32_t lo[D], hi[D];
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      lo[d] = INT32_MAX;
+      hi[d] = INT32_MIN;
+    }
+    const int64_t slot0 = g * a.C;
+    for (int s = lane; s < cnt; s += 32) {
+      const int64_t v = vals[b + s];
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        const int32_t c = a.pts[v * D + d];
+        a.pool.px[d][slot0 + s] = c;
+        lo[d] = min(lo[d], c);
+        hi[d] = max(hi[d], c);
+      }
+      a.pool.pid[slot0 + s] = a.ids[v];
+      a.pool.pkey[slot0 + s] = keys[b + s];
+    }
+#pragma unroll
+    for (int d = 0; d < D; ++d) {
+      lo[d] = __reduce_min_sync(0xFFFFFFFFu, lo[d]);
+      hi[d] = __reduce_max_sync(0xFFFFFFFFu, hi[d]);
+    }
+    if (lane == 0) {
+      const int64_t nd = a.node_off[ix] + j;
+#pragma unroll
+      for (int d = 0; d < D; ++d) {
+        a.nodes.lo[d][nd] = lo[d];
+        a.nodes.hi[d][nd] = hi[d];
+      }
+      a.nodes.cnt[nd] = cnt;
+      a.nodes.ref[nd] = (uint32_t)slot0;
+      a.nodes.kids[nd] = 0;
+      a.nodes.depth[nd] = 0;
+    }
+  }
+}
+
+// Summary levels: a block per index.
+template <int D>
+__global__ __launch_bounds__(512) void k_wide_summary(BuildArgs a) {
+  for (int ix = blockIdx.x; ix < a.nidx; ix += gridDim.x) {
+    const int64_t n = a.off[ix + 1] - a.off[ix];
+    if (n == 0) {
+      if (threadIdx.x == 0) a.root[ix] = -1;
+      continue;
+    }
+    const int64_t top = batch_summary<D>(a, a.node_off[ix], (n + a.phi - 1) / a.phi);
+    if (threadIdx.x == 0) a.root[ix] = (int32_t)top;
+  }
+}
+
+template <int D, int CURVE>
+psi_status build_wide(psi_batch *b, const BuildArgs &a, cudaStream_t s) {
+  const int64_t n = b->total;
+  auto grid = [&](int64_t items) { return (int)std::min<int64_t>(ceil_div(items, 256), (int64_t)num_sms() * 16); };
+  psi_status st;
+  SortResult r;
+  EncodeSpec none;
+  PSI_LAUNCH_NAMED("k_wide_keys", (k_wide_keys<D, CURVE>), grid(n), 256, 0, s, a.pts, n, a.bits, b->kA, b->vA, a.status);
+  if ((st = sort_pairs(none, b->kA, b->vA, n, 8, nullptr, b->kB, b->vB, b->kA, b->vA, a.status, s, &r))) return st;
+  const int low = std::max(b->key_bits - 8, 0);
+  PSI_LAUNCH(k_wide_segment, grid(n), 256, 0, s, b->d_off, b->nidx, low, r.vals, n, r.keys);
+  uint64_t *k0 = r.keys == b->kA ? b->kB : b->kA;
+  uint32_t *v0 = r.vals == b->vA ? b->vB : b->vA;
+  if ((st = sort_pairs(none, r.keys, r.vals, n, low + b->seg_bits, nullptr, k0, v0, r.keys, r.vals, a.status, s, &r)))
+    return st;
+  PSI_LAUNCH_NAMED("k_wide_full", (k_wide_full<D, CURVE>), grid(n), 256, 0, s, a.pts, r.vals, n, a.bits, r.keys);
+  // the sort's free key buffer lists the long runs (8 bytes per 33 positions)
+  int64_t *longs = reinterpret_cast<int64_t *>(r.keys == b->kA ? b->kB : b->kA);
+  PSI_CK(cudaMemsetAsync(b->d_nhard, 0, sizeof(uint32_t), s));
+  PSI_LAUNCH(k_wide_ties, grid(n), 256, 0, s, r.keys, r.vals, a.ids, b->d_off, b->nidx, n, longs, b->d_nhard);
+  PSI_LAUNCH(k_wide_tie_long, num_sms(), 1024, 0, s, r.keys, r.vals, a.ids, b->d_off, b->nidx, longs, b->d_nhard);
+  const int64_t leaves = b->block_off[b->nidx];
+  PSI_LAUNCH_NAMED("k_wide_gather", k_wide_gather<D>, (int)std::min<int64_t>(ceil_div(leaves, 8), (int64_t)num_sms() * 32),
+                   256, 0, s, r.keys, r.vals, a, leaves);
+  PSI_LAUNCH_NAMED("k_wide_summary", k_wide_summary<D>, std::min(b->nidx, num_sms() * 4), 512, 0, s, a);
+  PSI_CK(cudaGetLastError());
+  return PSI_OK;
 }
 
 // Root of each query's index; segment s covers queries [qoff[s], qoff[s+1]).
@@ -575,6 +801,17 @@ psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int
     set_error("batch too large for 32-bit node and slot references");
     return PSI_ERR_INVALID;
   }
+  // Device-wide, where the caller left the block's form open, when the largest index, or an even share of the points, keeps a
+  // block busy 1.3 times as long as the digit passes of the whole batch take
+  // (18 ns per point in a block; 0.013 ns per point and pass, and two passes'
+  // worth of gathers), and index numbers fit beside the keys.
+  while ((int64_t(1) << b->seg_bits) < nidx) ++b->seg_bits;
+  int64_t largest = 0;
+  for (int i = 0; i < nidx; ++i) largest = std::max(largest, b->off[i + 1] - b->off[i]);
+  const double passes = 1 + ceil_div(std::max(b->key_bits - 8, 0) + b->seg_bits, 8) + 2;
+  const double by_block = 18e-9 * (double)std::max<int64_t>(largest, b->total / num_sms());
+  b->wide = threads == 0 && cfg->radix_bits == 0 && b->total < (int64_t(1) << 30) && std::max(b->key_bits - 8, 0) + b->seg_bits <= 64 &&
+            by_block > 1.3 * (0.013e-9 * passes * (double)b->total + 200e-6);
   std::vector<int32_t> order(nidx);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
@@ -651,6 +888,7 @@ psi_status psi_batch_build(psi_batch *b, const int32_t *d_pts, const uint32_t *d
   a.status = b->d_status;
 #define BUILD_CASE(DD, CC)                                                        \
   do {                                                                            \
+    if (b->wide) return build_wide<DD, CC>(b, a, s);                              \
     if (b->rb == 11) {                                                            \
       if (b->threads == 256) return launch_build<DD, CC, 256, 11>(b, a, s);       \
       return launch_build<DD, CC, 512, 11>(b, a, s);                              \
