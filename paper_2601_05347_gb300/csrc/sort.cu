@@ -40,13 +40,25 @@ namespace psi {
 namespace {
 
 constexpr int ST = 256;        // threads per sort tile
-constexpr int SI = 16;         // keys per thread
+constexpr int SI = 16;         // keys per thread of a large sort
 constexpr int TILE = ST * SI;  // 4096 keys per tile
+// A pass of a sort of a few tiles takes one tile's latency (load, rank,
+// look-back, write: 12 us with 16 keys per thread), so a small sort takes
+// smaller tiles, and more predecessors per look-back step, until its longer
+// look-back chain costs more: per pass, with 16 / 4 keys per thread, 1e3 pairs
+// 12.3 / 8.2 us, 2e4 14.3 / 10.8, 6e4 14.8 / 13.1, 1.5e5 15.8 / 17.5 (8 keys per
+// thread: 3e5 16.4 / 20.6).
+constexpr int SI_SMALL = 4;
+constexpr int64_t kSmallSort = 80000;
 constexpr int SW = ST / 32;
 constexpr int MAX_PASSES = 8;  // 64-bit keys at 8-bit digits
 
 constexpr uint32_t LB_AGG = 1u << 30, LB_PRE = 2u << 30, LB_VAL = (1u << 30) - 1;
-constexpr int LB_W = 8;  // predecessor tiles read per look-back step
+// Predecessor tiles read per look-back step.  More read L2 faster than they save
+// steps in a large sort (1e8 pairs: 8 tiles 0.861 ms, 16 0.931); a small one's
+// chain is short and the words are all there.
+template <int KPT>
+constexpr int LB_W = KPT == SI ? 8 : 32;
 constexpr int HIST_U = 4;  // items per thread per round of the histogram pass
 
 // An event destroyed with its scope.
@@ -73,7 +85,7 @@ struct Radix {
   using Digit = typename std::conditional<RB == 8, uint8_t, uint16_t>::type;
 };
 
-template <int RB>
+template <int RB, int KPT = SI>
 struct OnesweepSmem {
   using R = Radix<RB>;
   typename R::Count wh[SW][R::RADIX];  // per-warp digit counters, then warp offsets
@@ -81,8 +93,8 @@ struct OnesweepSmem {
   uint32_t glob[R::RADIX];             // global position minus tile-local position
   uint32_t gb[R::RADIX];               // global exclusive digit offsets of this pass
   uint32_t nh[R::RADIX];               // next pass's digit counts of this tile
-  alignas(16) uint64_t stage[TILE];    // keys (then values) in digit order
-  typename R::Digit dig[TILE];         // digit of each staged position
+  alignas(16) uint64_t stage[ST * KPT];  // keys (then values) in digit order
+  typename R::Digit dig[ST * KPT];       // digit of each staged position
   uint32_t wsum[SW];
   alignas(16) uint8_t htab[kCurveTabBytes];
   uint32_t tile;
@@ -159,7 +171,8 @@ __device__ __forceinline__ uint64_t hll_hash(uint64_t x) {
 // keys are also written out (in input order) for the digit passes to read.  With 8-bit digits the counts go
 // to 4 shared copies (lane % 4 picks one) so that lanes of a warp hitting the
 // same digit -- common for the top digits of clustered input -- rarely collide.
-template <int MODE, int D, int CURVE, int RB>
+// BIG: enough points to pay for the larger curve tables.
+template <int MODE, int D, int CURVE, int RB, bool BIG>
 __global__ __launch_bounds__(256) void k_sort_hist(const uint64_t *kin, const int32_t *pts, int bits, int key_shift,
                                                    int64_t n, int passes, uint32_t *hist, int *status,
                                                    uint64_t *kst, unsigned long long *near, int near_shift,
@@ -173,8 +186,8 @@ __global__ __launch_bounds__(256) void k_sort_hist(const uint64_t *kin, const in
   uint8_t *htab = smem_raw + sizeof(uint32_t) * R::HIST_PARTS * (passes + 1) * R::RADIX;
   // Hilbert keys with larger tables than point_key's: 2D five levels per step
   // (8 KB), 3D two levels per step (13.5 KB)
-  constexpr bool H5 = MODE == 1 && D == 2 && CURVE == 1;
-  constexpr bool H3 = MODE == 1 && D == 3 && CURVE == 1;
+  constexpr bool H5 = BIG && MODE == 1 && D == 2 && CURVE == 1;
+  constexpr bool H3 = BIG && MODE == 1 && D == 3 && CURVE == 1;
   constexpr int TAB = H5 ? kHilbert5TabBytes : H3 ? kHilbert3x2TabBytes : kCurveTabBytes;
   uint32_t *shll = reinterpret_cast<uint32_t *>(htab + TAB);  // [kHllRegs] when ex.hll
   for (int i = threadIdx.x; i < R::HIST_PARTS * secs * R::RADIX; i += blockDim.x) shp[i] = 0;
@@ -309,12 +322,14 @@ __global__ void k_hist_scan(const uint32_t *hist, uint32_t *gbase) {
 
 // MODE 0: keys and values read; 1: keys computed from the points, values =
 // positions; 2: keys read, values = positions.
-template <int MODE, int D, int CURVE, int RB, int IO = IO_PAIRS>
-__global__ __launch_bounds__(ST, RB == 11 ? 2 : 3) void k_onesweep(PassArgs a) {
+template <int MODE, int D, int CURVE, int RB, int IO = IO_PAIRS, int SI = psi::SI>
+__global__ __launch_bounds__(ST, SI < psi::SI ? 4 : RB == 11 ? 2 : 3) void k_onesweep(PassArgs a) {
+  constexpr int TILE = ST * SI, LB_W = psi::LB_W<SI>;
   using R = Radix<RB>;
   constexpr int RADIX = R::RADIX, DPT = R::DPT;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  OnesweepSmem<RB> &sm = *reinterpret_cast<OnesweepSmem<RB> *>(smem_raw);
+  using Smem = OnesweepSmem<RB, SI>;
+  Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
 
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   if (tid == 0) sm.tile = atomicAdd(a.tile_ctr, 1u);
@@ -924,14 +939,14 @@ __global__ __launch_bounds__(1024) void k_prefix_long(uint64_t *keys, uint32_t *
 
 // ---------------------------------------------------------------------------
 
-template <int MODE, int D, int CURVE, int RB>
-static psi_status launch_hist(const uint64_t *kin, const EncodeSpec &enc, int64_t n, int passes, uint32_t *hist,
-                              int *status, cudaStream_t s, uint64_t *kst = nullptr,
-                              unsigned long long *near = nullptr, int near_shift = 0, HistExtra ex = HistExtra()) {
+template <int MODE, int D, int CURVE, int RB, bool BIG>
+static psi_status launch_hist_as(const uint64_t *kin, const EncodeSpec &enc, int64_t n, int passes, uint32_t *hist,
+                                 int *status, cudaStream_t s, uint64_t *kst, unsigned long long *near,
+                                 int near_shift, HistExtra ex) {
   using R = Radix<RB>;
-  auto kern = k_sort_hist<MODE, D, CURVE, RB>;
+  auto kern = k_sort_hist<MODE, D, CURVE, RB, BIG>;
   const size_t smem = sizeof(uint32_t) * R::HIST_PARTS * (passes + 1) * R::RADIX +
-                      (MODE == 1 && CURVE == 1 ? (D == 2 ? kHilbert5TabBytes : kHilbert3x2TabBytes)
+                      (BIG && MODE == 1 && CURVE == 1 ? (D == 2 ? kHilbert5TabBytes : kHilbert3x2TabBytes)
                                                : kCurveTabBytes) +
                       (ex.hll ? sizeof(uint32_t) * kHllRegs : 0);
   if (smem > 48 * 1024) PSI_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
@@ -944,13 +959,35 @@ static psi_status launch_hist(const uint64_t *kin, const EncodeSpec &enc, int64_
   return PSI_OK;
 }
 
-template <int MODE, int D, int CURVE, int RB, int IO = IO_PAIRS>
-static psi_status launch_pass(const PassArgs &a, int64_t tiles, cudaStream_t s) {
-  auto kern = k_onesweep<MODE, D, CURVE, RB, IO>;
-  const size_t smem = sizeof(OnesweepSmem<RB>);
+// Building the larger Hilbert tables takes a block about 2 us, as long as a
+// small sort's whole count.
+constexpr int64_t kBigTables = int64_t(1) << 18;
+
+template <int MODE, int D, int CURVE, int RB>
+static psi_status launch_hist(const uint64_t *kin, const EncodeSpec &enc, int64_t n, int passes, uint32_t *hist,
+                              int *status, cudaStream_t s, uint64_t *kst = nullptr,
+                              unsigned long long *near = nullptr, int near_shift = 0, HistExtra ex = HistExtra()) {
+  if (MODE == 1 && CURVE == 1 && n < kBigTables)
+    return launch_hist_as<MODE, D, CURVE, RB, false>(kin, enc, n, passes, hist, status, s, kst, near, near_shift, ex);
+  return launch_hist_as<MODE, D, CURVE, RB, true>(kin, enc, n, passes, hist, status, s, kst, near, near_shift, ex);
+}
+
+template <int MODE, int D, int CURVE, int RB, int IO = IO_PAIRS, int KPT = SI>
+static psi_status launch_pass_as(const PassArgs &a, int64_t tiles, cudaStream_t s) {
+  auto kern = k_onesweep<MODE, D, CURVE, RB, IO, KPT>;
+  const size_t smem = sizeof(OnesweepSmem<RB, KPT>);
   if (smem > 48 * 1024) PSI_CK(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   PSI_LAUNCH_NAMED("k_onesweep", kern, (unsigned)tiles, ST, smem, s, a);
   return PSI_OK;
+}
+
+// kpt: keys per thread (SI, or the smaller tiles of 8-bit sorts of pairs).
+template <int MODE, int D, int CURVE, int RB, int IO = IO_PAIRS>
+static psi_status launch_pass(const PassArgs &a, int64_t tiles, cudaStream_t s, int kpt = SI) {
+  if constexpr (RB == 8 && IO == IO_PAIRS) {
+    if (kpt == SI_SMALL) return launch_pass_as<MODE, D, CURVE, RB, IO, SI_SMALL>(a, tiles, s);
+  }
+  return launch_pass_as<MODE, D, CURVE, RB, IO>(a, tiles, s);
 }
 
 // The passes of a packed sort (8-bit digits only).
@@ -998,7 +1035,8 @@ static psi_status sort_pairs_rb(const EncodeSpec &enc, const uint64_t *keys_in, 
   using R = Radix<RB>;
   const bool encode = enc.pts != nullptr;
   const int passes_full = (key_bits + RB - 1) / RB;
-  const int64_t tiles = ceil_div(n, TILE);
+  const int kpt = RB == 8 && n <= kSmallSort ? SI_SMALL : SI;
+  const int64_t tiles = ceil_div(n, (int64_t)ST * kpt);
   // Decisions taken on the host from counts of the histogram pass are not
   // possible while the stream is being captured.
   cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -1016,16 +1054,18 @@ static psi_status sort_pairs_rb(const EncodeSpec &enc, const uint64_t *keys_in, 
   const bool pref_cand = may_prefix && encode && RB == 8 && n >= kPrefixMin && low_c > 0 &&
                          (key_bits - low_c + RB - 1) / RB < passes_full && !capturing;
   const bool pack_cand = encode && RB == 8 && n >= kPackMin && !capturing;
-  Buf<uint32_t> hist, lookback, ctr;
+  Buf<uint32_t> scratch;
   psi_status st;
   // digit counts: a section per pass, then the prefix sort's first digit;
   // two look-back tables used alternately: pass p clears the table of pass p+1
-  if ((st = hist.alloc((size_t)(passes_full + 1) * R::RADIX, s)) ||
-      (st = lookback.alloc((size_t)2 * tiles * R::RADIX, s)) || (st = ctr.alloc(passes_full, s)))
-    return st;
-  PSI_CK(cudaMemsetAsync(hist.p, 0, sizeof(uint32_t) * (passes_full + 1) * R::RADIX, s));
-  PSI_CK(cudaMemsetAsync(lookback.p, 0, sizeof(uint32_t) * tiles * R::RADIX, s));
-  PSI_CK(cudaMemsetAsync(ctr.p, 0, sizeof(uint32_t) * passes_full, s));
+  // (one allocation: counts, tile counters, the two tables; all but the second
+  // table start at zero)
+  const size_t n_hist = (size_t)(passes_full + 1) * R::RADIX, n_look = (size_t)tiles * R::RADIX;
+  if ((st = scratch.alloc(n_hist + R::RADIX + 2 * n_look, s))) return st;
+  struct {
+    uint32_t *p;
+  } hist{scratch.p}, ctr{scratch.p + n_hist}, lookback{scratch.p + n_hist + R::RADIX};
+  PSI_CK(cudaMemsetAsync(scratch.p, 0, sizeof(uint32_t) * (n_hist + R::RADIX + n_look), s));
 
   // Hilbert keys cost more arithmetic than their 8-byte write and read: the
   // histogram pass computes them once and writes them out; the first digit
@@ -1163,13 +1203,13 @@ static psi_status sort_pairs_rb(const EncodeSpec &enc, const uint64_t *keys_in, 
     if (p >= pk)
       st = launch_packed<RB>(enc, a, tiles, p == pk ? IO_PACK : (p + 1 < passes ? IO_KEYS : IO_UNPACK), s);
     else if (p > 0 || !encode)
-      st = launch_pass<0, 2, 0, RB>(a, tiles, s);
+      st = launch_pass<0, 2, 0, RB>(a, tiles, s, kpt);
     else if (stored)  // written keys, values = positions
-      st = launch_pass<2, 2, 0, RB>(a, tiles, s);
+      st = launch_pass<2, 2, 0, RB>(a, tiles, s, kpt);
     else if (enc.dim == 2)  // Morton keys computed from the points
-      st = launch_pass<1, 2, 0, RB>(a, tiles, s);
+      st = launch_pass<1, 2, 0, RB>(a, tiles, s, kpt);
     else
-      st = launch_pass<1, 3, 0, RB>(a, tiles, s);
+      st = launch_pass<1, 3, 0, RB>(a, tiles, s, kpt);
     if (st) return st;
   }
   out->keys = kb[(passes - 1) & 1];
