@@ -29,6 +29,16 @@ int64_t summary_capacity(int64_t L, int F);
 
 namespace {
 
+// Leaves a warp of the leaf kernels takes: 32 (one lane per leaf finds the
+// touched ones, the warp then works on each) where that leaves enough warps to
+// fill the chip, else fewer, for the warp works through its touched leaves one
+// after another (625 leaves, all touched: delete 57 -> 13 us).
+int leaves_per_warp(int64_t L) {
+  int w = 32;
+  while (w > 1 && ceil_div(L, w) < (int64_t)num_sms() * 48) w /= 2;
+  return w;
+}
+
 struct Batch {
   Buf<uint64_t> k0, k1;
   Buf<uint32_t> v0, v1;
@@ -149,11 +159,11 @@ __device__ __forceinline__ void sort_leaf_block(Pool &pool, uint32_t s0, int cnt
 // warp sorts each of those.
 template <int D>
 __global__ void k_sort_overflow_leaves(const int32_t *ncnt, const uint32_t *nref, const int32_t *sbeg,
-                                       const int32_t *send, int64_t L, int C, Pool pool) {
+                                       const int32_t *send, int64_t L, int C, Pool pool, int lpw) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; j0 < L; j0 += warps * 32) {
-    const int64_t jl = j0 + lane;
+  for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * lpw; j0 < L; j0 += warps * lpw) {
+    const int64_t jl = lane < lpw ? j0 + lane : L;
     uint32_t todo = __ballot_sync(0xFFFFFFFFu, jl < L && send[jl] > sbeg[jl] && ncnt[jl] + (send[jl] - sbeg[jl]) > C);
     while (todo) {
       const int64_t j = j0 + __ffs(todo) - 1;
@@ -224,6 +234,7 @@ struct InsertArgs {
   const int64_t *pos, *boff;
   int64_t L, Lnew;
   int64_t base_block;
+  int lpw;  // new leaves per warp
   const uint64_t *bkeys;
   const uint32_t *rid;  // batch records (k_batch_records): id and point of each sorted entry
   const int32_t *rpt;
@@ -243,10 +254,10 @@ template <int D>
 __global__ void k_insert_apply(InsertArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t o0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; o0 < a.Lnew; o0 += warps * 32) {
+  for (int64_t o0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * a.lpw; o0 < a.Lnew; o0 += warps * a.lpw) {
     bool touched = false;
     {
-      const int64_t ol = o0 + lane;
+      const int64_t ol = lane < a.lpw ? o0 + lane : a.Lnew;
       if (ol < a.Lnew) {
         const int64_t j = a.owner[ol];
         if (a.send[j] == a.sbeg[j]) {
@@ -397,11 +408,11 @@ __global__ void k_insert_apply(InsertArgs a) {
 // leaves, one lane per leaf finds those with a slice.
 template <int D>
 __global__ void k_append_inplace(Leaves lv, Pool pool, const int32_t *sbeg, const int32_t *send, int64_t L,
-                                 const uint64_t *bkeys, const uint32_t *rid, const int32_t *rpt) {
+                                 const uint64_t *bkeys, const uint32_t *rid, const int32_t *rpt, int lpw) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; j0 < L; j0 += warps * 32) {
-    const int64_t jl = j0 + lane;
+  for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * lpw; j0 < L; j0 += warps * lpw) {
+    const int64_t jl = lane < lpw ? j0 + lane : L;
     uint32_t todo = __ballot_sync(0xFFFFFFFFu, jl < L && send[jl] > sbeg[jl]);
     while (todo) {
       const int64_t j = j0 + __ffs(todo) - 1;
@@ -468,12 +479,12 @@ constexpr int DG = 2;
 template <int D, int R>
 __global__ void k_delete_leaves(Leaves lv, Pool pool, const int32_t *sbeg, const int32_t *send, int64_t L,
                                 const uint64_t *bkeys, const uint32_t *rid, const int32_t *rpt,
-                                unsigned long long *deleted) {
+                                unsigned long long *deleted, int lpw) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
   uint32_t removed = 0;  // lane 0: points this warp removed
-  for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; j0 < L; j0 += warps * 32) {
-    const int64_t jl = j0 + lane;
+  for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * lpw; j0 < L; j0 += warps * lpw) {
+    const int64_t jl = lane < lpw ? j0 + lane : L;
     uint32_t todo = __ballot_sync(0xFFFFFFFFu, jl < L && send[jl] > sbeg[jl]);
     while (todo) {
       int64_t j[DG];
@@ -635,11 +646,11 @@ __global__ void k_wrap_plan(const int32_t *cnt, const int32_t *start, const int6
 // leaf order are then sorted by (key, id) as a whole).
 template <int D>
 __global__ void k_sort_flagged_leaves(const int32_t *cnt, const uint32_t *ref, const int32_t *flag, int64_t L,
-                                      Pool pool) {
+                                      Pool pool, int lpw) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; j0 < L; j0 += warps * 32) {
-    const int64_t jl = j0 + lane;
+  for (int64_t j0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * lpw; j0 < L; j0 += warps * lpw) {
+    const int64_t jl = lane < lpw ? j0 + lane : L;
     uint32_t todo = __ballot_sync(0xFFFFFFFFu, jl < L && flag[jl] && cnt[jl] > 1);
     while (todo) {
       const int64_t j = j0 + __ffs(todo) - 1;
@@ -655,7 +666,7 @@ struct WrapArgs {
   const int32_t *owner, *start, *ge, *outl;
   const int64_t *gx, *pos, *boff, *E;
   int64_t Lnew, base_block;
-  int C;
+  int C, lpw;
 };
 
 // A warp takes 32 new leaf positions: a lane copies the descriptor of a kept
@@ -664,10 +675,10 @@ template <int D>
 __global__ void k_wrap_apply(WrapArgs a) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t o0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * 32; o0 < a.Lnew; o0 += warps * 32) {
+  for (int64_t o0 = (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * a.lpw; o0 < a.Lnew; o0 += warps * a.lpw) {
     bool part = false;
     {
-      const int64_t ol = o0 + lane;
+      const int64_t ol = lane < a.lpw ? o0 + lane : a.Lnew;
       if (ol < a.Lnew) {
         const int64_t j = a.owner[ol];
         if (!a.start[j]) {
@@ -828,14 +839,15 @@ psi_status spac_insert(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
   PSI_CK(cudaStreamSynchronize(s));
   const int64_t Lnew = h[0], NB = h[1];
 
+  const int lpw = leaves_per_warp(L);
   if (NB == 0) {  // no leaf overflows: append in place, the leaf list keeps its shape
     Leaves lv = leaves_of(ix->nodes, ix->sep_key, ix->sep_id);
     if (ix->D == 2)
-      PSI_LAUNCH_NAMED("k_append_inplace", k_append_inplace<2>, warp_grid(ceil_div(L, 32)), 256, 0, s, lv, ix->pool,
-                       sbeg.p, send.p, L, b.keys, rid.p, rpt.p);
+      PSI_LAUNCH_NAMED("k_append_inplace", k_append_inplace<2>, warp_grid(ceil_div(L, lpw)), 256, 0, s, lv, ix->pool,
+                       sbeg.p, send.p, L, b.keys, rid.p, rpt.p, lpw);
     else
-      PSI_LAUNCH_NAMED("k_append_inplace", k_append_inplace<3>, warp_grid(ceil_div(L, 32)), 256, 0, s, lv, ix->pool,
-                       sbeg.p, send.p, L, b.keys, rid.p, rpt.p);
+      PSI_LAUNCH_NAMED("k_append_inplace", k_append_inplace<3>, warp_grid(ceil_div(L, lpw)), 256, 0, s, lv, ix->pool,
+                       sbeg.p, send.p, L, b.keys, rid.p, rpt.p, lpw);
     ix->n += m;
     if ((st = build_spac_summary(ix, s))) return st;
     PSI_CK(cudaGetLastError());
@@ -845,11 +857,11 @@ psi_status spac_insert(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
   const int64_t base_block = ix->pool_used;
   if ((st = grow_pool(ix, (base_block + NB) * ix->C, base_block * ix->C, s))) return st;
   if (ix->D == 2)
-    PSI_LAUNCH_NAMED("k_sort_overflow_leaves", k_sort_overflow_leaves<2>, warp_grid(ceil_div(L, 32)), 256, 0, s,
-                     ix->nodes.cnt, ix->nodes.ref, sbeg.p, send.p, L, ix->C, ix->pool);
+    PSI_LAUNCH_NAMED("k_sort_overflow_leaves", k_sort_overflow_leaves<2>, warp_grid(ceil_div(L, lpw)), 256, 0, s,
+                     ix->nodes.cnt, ix->nodes.ref, sbeg.p, send.p, L, ix->C, ix->pool, lpw);
   else
-    PSI_LAUNCH_NAMED("k_sort_overflow_leaves", k_sort_overflow_leaves<3>, warp_grid(ceil_div(L, 32)), 256, 0, s,
-                     ix->nodes.cnt, ix->nodes.ref, sbeg.p, send.p, L, ix->C, ix->pool);
+    PSI_LAUNCH_NAMED("k_sort_overflow_leaves", k_sort_overflow_leaves<3>, warp_grid(ceil_div(L, lpw)), 256, 0, s,
+                     ix->nodes.cnt, ix->nodes.ref, sbeg.p, send.p, L, ix->C, ix->pool, lpw);
 
   NodeArrays na;
   uint64_t *nsk = nullptr;
@@ -884,15 +896,16 @@ psi_status spac_insert(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
   a.L = L;
   a.Lnew = Lnew;
   a.base_block = base_block;
+  a.lpw = leaves_per_warp(Lnew);
   a.bkeys = b.keys;
   a.rid = rid.p;
   a.rpt = rpt.p;
   a.C = ix->C;
   a.phi = ix->phi;
   if (ix->D == 2)
-    PSI_LAUNCH_NAMED("k_insert_apply", k_insert_apply<2>, warp_grid(ceil_div(Lnew, 32)), 256, 0, s, a);
+    PSI_LAUNCH_NAMED("k_insert_apply", k_insert_apply<2>, warp_grid(ceil_div(Lnew, a.lpw)), 256, 0, s, a);
   else
-    PSI_LAUNCH_NAMED("k_insert_apply", k_insert_apply<3>, warp_grid(ceil_div(Lnew, 32)), 256, 0, s, a);
+    PSI_LAUNCH_NAMED("k_insert_apply", k_insert_apply<3>, warp_grid(ceil_div(Lnew, a.lpw)), 256, 0, s, a);
   free_nodes(ix->nodes, s);
   DevMem::free(ix->sep_key, s);
   DevMem::free(ix->sep_id, s);
@@ -928,21 +941,22 @@ psi_status spac_delete(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
   Buf<int32_t> rpt;
   if ((st = batch_records(ix, b, pts, ids, m, s, rid, rpt))) return st;
   Leaves lv = leaves_of(ix->nodes, ix->sep_key, ix->sep_id);
-  const int g = warp_grid(ceil_div(L, 32));
+  const int lpw = leaves_per_warp(L);
+  const int g = warp_grid(ceil_div(L, lpw));
   if (ix->D == 2) {
     if (ix->C <= 64)
       PSI_LAUNCH_NAMED("k_delete_leaves", (k_delete_leaves<2, 2>), g, 256, 0, s, lv, ix->pool, sbeg.p, send.p, L,
-                       b.keys, rid.p, rpt.p, del.p);
+                       b.keys, rid.p, rpt.p, del.p, lpw);
     else
       PSI_LAUNCH_NAMED("k_delete_leaves", (k_delete_leaves<2, MAXPL>), g, 256, 0, s, lv, ix->pool, sbeg.p, send.p, L,
-                       b.keys, rid.p, rpt.p, del.p);
+                       b.keys, rid.p, rpt.p, del.p, lpw);
   } else {
     if (ix->C <= 64)
       PSI_LAUNCH_NAMED("k_delete_leaves", (k_delete_leaves<3, 2>), g, 256, 0, s, lv, ix->pool, sbeg.p, send.p, L,
-                       b.keys, rid.p, rpt.p, del.p);
+                       b.keys, rid.p, rpt.p, del.p, lpw);
     else
       PSI_LAUNCH_NAMED("k_delete_leaves", (k_delete_leaves<3, MAXPL>), g, 256, 0, s, lv, ix->pool, sbeg.p, send.p, L,
-                       b.keys, rid.p, rpt.p, del.p);
+                       b.keys, rid.p, rpt.p, del.p, lpw);
   }
   // the leaf wrap (Sec 4.2): runs of leaves left below h points join the leaf
   // after them and are re-wrapped
@@ -982,11 +996,11 @@ psi_status spac_delete(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
   const int64_t base_block = ix->pool_used;
   if ((st = grow_pool(ix, (base_block + NB) * ix->C, base_block * ix->C, s))) return st;
   if (ix->D == 2)
-    PSI_LAUNCH_NAMED("k_sort_flagged_leaves", k_sort_flagged_leaves<2>, warp_grid(ceil_div(L, 32)), 256, 0, s,
-                     ix->nodes.cnt, ix->nodes.ref, ingroup.p, L, ix->pool);
+    PSI_LAUNCH_NAMED("k_sort_flagged_leaves", k_sort_flagged_leaves<2>, warp_grid(ceil_div(L, lpw)), 256, 0, s,
+                     ix->nodes.cnt, ix->nodes.ref, ingroup.p, L, ix->pool, lpw);
   else
-    PSI_LAUNCH_NAMED("k_sort_flagged_leaves", k_sort_flagged_leaves<3>, warp_grid(ceil_div(L, 32)), 256, 0, s,
-                     ix->nodes.cnt, ix->nodes.ref, ingroup.p, L, ix->pool);
+    PSI_LAUNCH_NAMED("k_sort_flagged_leaves", k_sort_flagged_leaves<3>, warp_grid(ceil_div(L, lpw)), 256, 0, s,
+                     ix->nodes.cnt, ix->nodes.ref, ingroup.p, L, ix->pool, lpw);
   NodeArrays na;
   uint64_t *nsk = nullptr;
   uint32_t *nsi = nullptr;
@@ -1023,10 +1037,11 @@ psi_status spac_delete(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
     a.Lnew = Lnew;
     a.base_block = base_block;
     a.C = ix->C;
+    a.lpw = leaves_per_warp(Lnew);
     if (ix->D == 2)
-      PSI_LAUNCH_NAMED("k_wrap_apply", k_wrap_apply<2>, warp_grid(ceil_div(Lnew, 32)), 256, 0, s, a);
+      PSI_LAUNCH_NAMED("k_wrap_apply", k_wrap_apply<2>, warp_grid(ceil_div(Lnew, a.lpw)), 256, 0, s, a);
     else
-      PSI_LAUNCH_NAMED("k_wrap_apply", k_wrap_apply<3>, warp_grid(ceil_div(Lnew, 32)), 256, 0, s, a);
+      PSI_LAUNCH_NAMED("k_wrap_apply", k_wrap_apply<3>, warp_grid(ceil_div(Lnew, a.lpw)), 256, 0, s, a);
   }
   free_nodes(ix->nodes, s);
   DevMem::free(ix->sep_key, s);
