@@ -204,48 +204,57 @@ __device__ __forceinline__ void klist_fill(KList<KPL, int64_t> &kl, bool in, int
   kl.refresh_kth(k);
 }
 
-// Offers one candidate per lane (`in`: it beats the current k-th).  With more
-// than six entrants they are sorted across the warp and merged into the list
-// row by row: the row against the reversed carry gives, lane-wise, the 32
-// smallest of both (a bitonic sequence, cleaned into the row) and the 32
-// largest (cleaned into the carry for the next row); otherwise the entrants
-// are inserted one at a time.
+// Merges one candidate per lane (absent: +inf) into the list: sorted across the
+// warp, then row by row: the row against the reversed carry gives, lane-wise,
+// the 32 smallest of both (a bitonic sequence, cleaned into the row) and the 32
+// largest (cleaned into the carry for the next row).  A row whose last entry
+// precedes every candidate is passed by.
 template <int KPL, typename T>
-__device__ __forceinline__ void klist_offer(KList<KPL, T> &kl, bool in, T d2, uint32_t id, int k) {
+__device__ __forceinline__ void klist_merge(KList<KPL, T> &kl, T cd, uint32_t ci, int k) {
   const int lane = threadIdx.x & 31;
-  uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
-  if (__popc(m) > 6) {
-    T cd = in ? d2 : DistInf<T>::v();
-    uint32_t ci = in ? id : 0xFFFFFFFFu;
-    warp_sort_pairs(cd, ci);
+  warp_sort_pairs(cd, ci);
 #pragma unroll
-    for (int r = 0; r < KPL; ++r) {
-      if (__ballot_sync(0xFFFFFFFFu, cd != DistInf<T>::v()) == 0) break;  // nothing left to place
-      const T rd = __shfl_sync(0xFFFFFFFFu, cd, 31 - lane);
-      const uint32_t ri = __shfl_sync(0xFFFFFFFFu, ci, 31 - lane);
-      T lo_d = kl.d[r], hi_d = rd;
-      uint32_t lo_i = kl.i[r], hi_i = ri;
-      if (pair_less(rd, ri, lo_d, lo_i)) {
-        hi_d = lo_d;
-        hi_i = lo_i;
-        lo_d = rd;
-        lo_i = ri;
-      }
-      warp_bitonic_clean(lo_d, lo_i);
+  for (int r = 0; r < KPL; ++r) {
+    const T fd = __shfl_sync(0xFFFFFFFFu, cd, 0);
+    const uint32_t fi = __shfl_sync(0xFFFFFFFFu, ci, 0);
+    if (fd == DistInf<T>::v()) break;  // nothing left to place
+    if (KPL > 1 && __any_sync(0xFFFFFFFFu, lane == 31 && pair_less(kl.d[r], kl.i[r], fd, fi))) continue;
+    const T rd = __shfl_sync(0xFFFFFFFFu, cd, 31 - lane);
+    const uint32_t ri = __shfl_sync(0xFFFFFFFFu, ci, 31 - lane);
+    T lo_d = kl.d[r], hi_d = rd;
+    uint32_t lo_i = kl.i[r], hi_i = ri;
+    if (pair_less(rd, ri, lo_d, lo_i)) {
+      hi_d = lo_d;
+      hi_i = lo_i;
+      lo_d = rd;
+      lo_i = ri;
+    }
+    warp_bitonic_clean(lo_d, lo_i);
+    kl.d[r] = lo_d;
+    kl.i[r] = lo_i;
+    if (r + 1 < KPL) {
       warp_bitonic_clean(hi_d, hi_i);
-      kl.d[r] = lo_d;
-      kl.i[r] = lo_i;
       cd = hi_d;
       ci = hi_i;
     }
-    // entries past the k-th are dropped; the k-th bounds admission
+  }
+  // entries past the k-th are dropped; the k-th bounds admission
 #pragma unroll
-    for (int r = 0; r < KPL; ++r)
-      if (r * 32 + lane >= k) {
-        kl.d[r] = DistInf<T>::v();
-        kl.i[r] = 0xFFFFFFFFu;
-      }
-    kl.refresh_kth(k);
+  for (int r = 0; r < KPL; ++r)
+    if (r * 32 + lane >= k) {
+      kl.d[r] = DistInf<T>::v();
+      kl.i[r] = 0xFFFFFFFFu;
+    }
+  kl.refresh_kth(k);
+}
+
+// Offers one candidate per lane (`in`: it beats the current k-th): more than six
+// are merged at once, fewer inserted one at a time.
+template <int KPL, typename T>
+__device__ __forceinline__ void klist_offer(KList<KPL, T> &kl, bool in, T d2, uint32_t id, int k) {
+  uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+  if (__popc(m) > 6) {
+    klist_merge(kl, in ? d2 : DistInf<T>::v(), in ? id : 0xFFFFFFFFu, k);
     return;
   }
   while (m) {
@@ -255,6 +264,42 @@ __device__ __forceinline__ void klist_offer(KList<KPL, T> &kl, bool in, T d2, ui
     const uint32_t ci = __shfl_sync(0xFFFFFFFFu, id, src);
     if (kl.admits(cd, ci)) kl.insert(cd, ci, k);
   }
+}
+
+// Candidates of a long list (KPL > 1) waiting in shared memory: merging 32 of
+// them costs little more than merging seven, so they are collected over leaves
+// and merged when there are 32 (or at klist_flush).
+struct KWait {
+  int64_t d[64];
+  uint32_t i[64];
+};
+
+template <int KPL>
+__device__ __forceinline__ void klist_flush(KList<KPL> &kl, KWait &wt, int &nw, int k) {
+  const int lane = threadIdx.x & 31;
+  __syncwarp();
+  const bool in = lane < min(nw, 32);
+  klist_merge(kl, in ? wt.d[lane] : INT64_MAX, in ? wt.i[lane] : 0xFFFFFFFFu, k);
+  const int left = max(nw - 32, 0);
+  if (lane < left) {
+    wt.d[lane] = wt.d[lane + 32];
+    wt.i[lane] = wt.i[lane + 32];
+  }
+  __syncwarp();
+  nw = left;
+}
+
+// nw: candidates waiting (at most 31 between calls).
+template <int KPL>
+__device__ __forceinline__ void klist_wait(KList<KPL> &kl, KWait &wt, int &nw, bool in, int64_t d2, uint32_t id, int k) {
+  const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
+  if (in) {
+    const int p = nw + __popc(m & ((1u << (threadIdx.x & 31)) - 1u));
+    wt.d[p] = d2;
+    wt.i[p] = id;
+  }
+  nw += __popc(m);
+  if (nw >= 32) klist_flush(kl, wt, nw, k);
 }
 
 // ---- pairs in one thread's registers (the one-query-per-thread kernels) -------

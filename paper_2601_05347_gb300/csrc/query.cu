@@ -76,7 +76,7 @@ __device__ __forceinline__ int box_relation(const TreeView &t, uint32_t node, co
 // EMPTY: the list is known to be empty (the first leaf a query scans).
 template <int D, int KPL, bool EMPTY = false>
 __device__ __forceinline__ void knn_scan_slots(const TreeView &t, uint32_t s0, int cnt, const int32_t *qc,
-                                               KList<KPL> &kl, int k) {
+                                               KList<KPL> &kl, KWait *wt, int &nw, int k) {
   const int lane = threadIdx.x & 31;
   for (int b = 0; b < cnt; b += 32) {
     const int s = b + lane;
@@ -97,6 +97,8 @@ __device__ __forceinline__ void knn_scan_slots(const TreeView &t, uint32_t s0, i
     }
     if (EMPTY && b == 0)  // the list holds nothing yet: every point enters
       klist_fill(kl, valid, d2, id, k);
+    else if constexpr (KPL > 1)
+      klist_wait(kl, *wt, nw, valid && kl.admits(d2, id), d2, id, k);
     else
       klist_offer(kl, valid && kl.admits(d2, id), d2, id, k);
   }
@@ -104,8 +106,8 @@ __device__ __forceinline__ void knn_scan_slots(const TreeView &t, uint32_t s0, i
 
 template <int D, int KPL, bool EMPTY = false>
 __device__ __forceinline__ void knn_scan_leaf(const TreeView &t, uint32_t node, const int32_t *qc, KList<KPL> &kl,
-                                              int k) {
-  knn_scan_slots<D, KPL, EMPTY>(t, t.ref[node], t.cnt[node], qc, kl, k);
+                                              KWait *wt, int &nw, int k) {
+  knn_scan_slots<D, KPL, EMPTY>(t, t.ref[node], t.cnt[node], qc, kl, wt, nw, k);
 }
 
 struct KnnStats {
@@ -190,8 +192,10 @@ template <int D, int KPL, bool STATS, bool BATCH, bool LIST = false, bool SELF =
 __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
   // internal nodes still to visit: (node, key, first child, children)
   __shared__ uint4 s_stk[QW][KSTACK];
+  __shared__ KWait s_wait[KPL > 1 ? QW : 1];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int64_t nw = (int64_t)gridDim.x * QW;
+  KWait *wt = &s_wait[KPL > 1 ? w : 0];
+  const int64_t warps = (int64_t)gridDim.x * QW;
   const int64_t nq = LIST ? (int64_t)*a.d_nq : a.nq;
   const TreeView &t = a.t;
   __shared__ alignas(16) uint8_t s_tab[SELF ? kCurveTabBytes : 16];
@@ -200,13 +204,14 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
     __syncthreads();
   }
   unsigned long long n_int = 0, n_leaf = 0, n_pts = 0, n_kids = 0;
-  for (int64_t qi = (int64_t)blockIdx.x * QW + w; qi < nq; qi += nw) {
+  for (int64_t qi = (int64_t)blockIdx.x * QW + w; qi < nq; qi += warps) {
     const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
     int32_t qc[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) qc[d] = a.q[q * D + d];
     KList<KPL> kl;
     kl.init();
+    int nw = 0;  // candidates waiting
     const int32_t root = a.qroot ? a.qroot[q] : t.root;
     // seed leaves [s_lo, s_hi]: the leaf at the query's curve position, widened
     // along the curve until it holds at least k points
@@ -223,14 +228,14 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
       const uint64_t key = sd.curve == CURVE_HILBERT ? point_key<D, CURVE_HILBERT>(s_tab, qc, sd.self_bits, bad)
                                                      : point_key<D, CURVE_MORTON>(s_tab, qc, sd.self_bits, bad);
       s_lo = s_hi = seed_search_warp(sd.sep_key, sd.L, key);
-      knn_scan_leaf<D, KPL, true>(t, (uint32_t)s_lo, qc, kl, a.k);
+      knn_scan_leaf<D, KPL, true>(t, (uint32_t)s_lo, qc, kl, wt, nw, a.k);
     } else if (sd.qkey && root >= 0) {
       const int64_t pos = sd.pos[qi];  // k_knn_seed
       if (L > 0) {
         // P-Orth: pos is a position in the key-ordered leaf list
         const int64_t j = sd.leaf_node ? (int64_t)sd.leaf_node[pos] : pos;
         const int64_t le = lb + L;
-        knn_scan_leaf<D, KPL, true>(t, (uint32_t)j, qc, kl, a.k);
+        knn_scan_leaf<D, KPL, true>(t, (uint32_t)j, qc, kl, wt, nw, a.k);
         int64_t got = t.cnt[j];
         if (STATS) {
           ++n_leaf;
@@ -247,7 +252,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
             nx = ++s_hi;
           else
             nx = --s_lo;
-          knn_scan_leaf<D, KPL>(t, (uint32_t)nx, qc, kl, a.k);
+          knn_scan_leaf<D, KPL>(t, (uint32_t)nx, qc, kl, wt, nw, a.k);
           got += t.cnt[nx];
           if (STATS) {
             ++n_leaf;
@@ -259,6 +264,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
     // seed leaves as a node range [slo, shi] (empty: slo > shi)
     const uint32_t slo = s_hi < s_lo ? 1u : (uint32_t)s_lo;
     const uint32_t shi = s_hi < s_lo ? 0u : (uint32_t)s_hi;
+    if (KPL > 1 && nw) klist_flush(kl, *wt, nw, a.k);
     uint32_t kdk = order_key(kl.kd);
     int sp = 0;
     // Children [c0, c0 + nk) of an expanded node: the internal ones that may
@@ -348,7 +354,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
           ml &= ~(1u << src);
           const uint32_t lref = __shfl_sync(0xFFFFFFFFu, cref, src);
           const int lcnt = __shfl_sync(0xFFFFFFFFu, ccnt, src);
-          knn_scan_slots<D, KPL>(t, lref, lcnt, qc, kl, a.k);
+          knn_scan_slots<D, KPL>(t, lref, lcnt, qc, kl, wt, nw, a.k);
           kdk = order_key(kl.kd);
           if (STATS) {
             ++n_leaf;
@@ -412,7 +418,10 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
               d2 += (int64_t)dd * dd;
             }
           }
-          klist_offer(kl, valid && kl.admits(d2, id), d2, id, a.k);
+          if constexpr (KPL > 1)
+            klist_wait(kl, *wt, nw, valid && kl.admits(d2, id), d2, id, a.k);
+          else
+            klist_offer(kl, valid && kl.admits(d2, id), d2, id, a.k);
         }
         kdk = order_key(kl.kd);
       }
@@ -420,7 +429,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
     if (root >= 0) {
       if (t.kids[root] == 0) {
         if (!((uint32_t)root >= slo && (uint32_t)root <= shi))
-          knn_scan_leaf<D, KPL>(t, (uint32_t)root, qc, kl, a.k);
+          knn_scan_leaf<D, KPL>(t, (uint32_t)root, qc, kl, wt, nw, a.k);
       } else {
         // the root as the first entry: one call site keeps `expand` inlined
         uint32_t c0 = t.ref[root], pkey = 0;
@@ -455,6 +464,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
         }
       }
     }
+    if (KPL > 1 && nw) klist_flush(kl, *wt, nw, a.k);
 #pragma unroll
     for (int r = 0; r < KPL; ++r) {
       const int e = r * 32 + lane;
