@@ -1193,6 +1193,13 @@ static int64_t lane_min_queries(int D, int k, bool porth) {
   return k <= 5 ? wave * 5 / 2 : wave * 4;
 }
 
+// On P-Orth, one query per warp with small leaves scanned together beats two
+// queries per warp with one leaf at a time, except where the lists are short
+// and there are many queries.  10-NN, two per warp / one, in us: 3D uniform 5e3
+// queries 257 / 108, 1e5 759 / 632 (32-NN 1473 / 937); 2D Varden 5e3 203 / 99,
+// 1e5 533 / 592 (32-NN 857 / 753).
+static bool porth_single(int D, int k, int64_t nq) { return k > (D == 3 ? 8 : 16) || (nq < 32768 && k > 4); }
+
 psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k, const uint32_t *order,
                          const int32_t *qroot, int D, uint32_t *out_id, int64_t *out_d2, int *status,
                          unsigned long long *d_stats, cudaStream_t s, const KnnSeed &seed, int64_t leaf_limit,
@@ -1219,7 +1226,7 @@ psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k
     a.d_nq = hard.n;
 #define KNN_LIST(DD, PP)                                                                                            \
   do {                                                                                                              \
-    if (qroot)                                                                                                      \
+    if (qroot || (porth && porth_single(D, k, nq)))                                                                  \
       PSI_LAUNCH_NAMED("k_knn", (k_knn<DD, 1, false, PP, true>),                                                    \
                        resident_query_grid(k_knn<DD, 1, false, PP, true>, nq), QW * 32, 0, s, a, stats);            \
     else                                                                                                            \
@@ -1240,7 +1247,7 @@ psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k
   }
   const int kpl = k <= 32 ? 1 : (k <= 64 ? 2 : 4);
   // k <= 32 over one tree with queries in curve order: kGroup queries per warp
-  if (kpl == 1 && !qroot && order && kGroup > 1) {
+  if (kpl == 1 && !qroot && order && kGroup > 1 && !(porth && porth_single(D, k, nq))) {
 #define KNN_GROUP(DD, RC)                                                                                   \
   do {                                                                                                      \
     if (d_stats)                                                                                            \
