@@ -935,6 +935,207 @@ __global__ __launch_bounds__(1024) void k_prefix_long(uint64_t *keys, uint32_t *
   }
 }
 
+// ---- Small encoding sorts: tiles sorted in registers, then ranked ----------------
+// Eight digit passes over a few tiles are eight launches that each take a
+// tile's latency.  An encoding sort of at most kRankSort points instead takes
+// two launches: every block computes the keys of 1024 points and sorts them by
+// (key, tie) with a bitonic network in registers (tie: the id where equal keys
+// are to be in id order, else the position), then every element finds its place
+// among each other tile's by binary search and writes itself there.  Equal
+// pairs (a batch may repeat an entry) keep the tiles' order.  Both launches are
+// bound by latency (one block per SM or few); the second's work grows with the
+// square of the points, hence the limit.  Whole 2D builds by digit passes / by
+// ranks: 1e3 points 129 / 76 us, 1.6e4 153 / 88, 6.4e4 180 / 131, 1e5 198 / 181,
+// 1.3e5 201 / 244.
+constexpr int RT = 256, RE = 4, RTILE = RT * RE;
+constexpr int64_t kRankSort = 81920;
+
+struct RankArrays {  // padded to whole tiles (key and tie all ones past the end)
+  uint64_t *key;
+  uint32_t *tie, *val;
+};
+
+// (ka, ta) < (kb, tb) as 96-bit numbers: the borrow of one subtraction, without
+// branches (with them the network took twice the instructions).
+__device__ __forceinline__ bool rank_less(uint64_t ka, uint32_t ta, uint64_t kb, uint32_t tb) {
+  uint32_t t, r;
+  asm("sub.cc.u32 %0, %2, %3;\n\t"
+      "subc.cc.u32 %0, %4, %5;\n\t"
+      "subc.cc.u32 %0, %6, %7;\n\t"
+      "subc.u32 %1, 0, 0;"
+      : "=&r"(t), "=r"(r)
+      : "r"(ta), "r"(tb), "r"((uint32_t)ka), "r"((uint32_t)kb), "r"((uint32_t)(ka >> 32)), "r"((uint32_t)(kb >> 32)));
+  (void)t;
+  return r != 0;
+}
+
+template <int D, int CURVE>
+__global__ __launch_bounds__(RT) void k_rank_tiles(EncodeSpec enc, const uint32_t *tie_ids, int64_t n, RankArrays out,
+                                                   int *status) {
+  __shared__ alignas(16) uint8_t htab[kCurveTabBytes];
+  __shared__ uint64_t sk[RTILE];
+  __shared__ uint32_t st[RTILE], sv[RTILE];
+  const int t = threadIdx.x;
+  curve_table_init<D, CURVE>(htab);
+  __syncthreads();
+  uint64_t k[RE];
+  uint32_t ti[RE], v[RE];
+  bool bad_any = false;
+#pragma unroll
+  for (int e = 0; e < RE; ++e) {
+    const int64_t i = (int64_t)blockIdx.x * RTILE + e * RT + t;
+    k[e] = ~0ull;
+    ti[e] = v[e] = 0xFFFFFFFFu;
+    if (i < n) {
+      int32_t c[D];
+#pragma unroll
+      for (int d = 0; d < D; ++d) c[d] = enc.pts[i * D + d];
+      bool bad;
+      // (a coordinate out of range is reported; its key stays below the padding's)
+      k[e] = (point_key<D, CURVE>(htab, c, enc.bits, bad) & ((uint64_t(1) << (D * enc.bits)) - 1)) >> enc.key_shift;
+      bad_any |= bad;
+      ti[e] = tie_ids ? tie_ids[i] : (uint32_t)i;
+      v[e] = (uint32_t)i;
+    }
+  }
+  if (bad_any) atomicOr(status, ST_RANGE);
+  // Value e of thread t stands at position t * RE + e.
+  auto take = [&](bool low, int e, uint64_t ok, uint32_t ot, uint32_t ov) {
+    // low keeps the smaller, else the larger; equal pairs stay
+    const bool sw = rank_less(ok, ot, k[e], ti[e]) == low && !(ok == k[e] && ot == ti[e]);
+    k[e] = sw ? ok : k[e];
+    ti[e] = sw ? ot : ti[e];
+    v[e] = sw ? ov : v[e];
+  };
+#pragma unroll 1
+  for (int kk = 2; kk <= RTILE; kk <<= 1) {
+    int j = kk >> 1;
+#pragma unroll 1
+    for (; j >= 32 * RE; j >>= 1) {
+      __syncthreads();
+#pragma unroll
+      for (int e = 0; e < RE; ++e) {
+        sk[e * RT + t] = k[e];
+        st[e * RT + t] = ti[e];
+        sv[e * RT + t] = v[e];
+      }
+      __syncthreads();
+      const int x = t ^ (j / RE);
+      const bool low = ((t & (j / RE)) == 0) == ((t * RE & kk) == 0);
+#pragma unroll
+      for (int e = 0; e < RE; ++e) take(low, e, sk[e * RT + x], st[e * RT + x], sv[e * RT + x]);
+    }
+#pragma unroll 1
+    for (; j >= RE; j >>= 1) {
+      const bool low = ((t & (j / RE)) == 0) == ((t * RE & kk) == 0);
+#pragma unroll
+      for (int e = 0; e < RE; ++e)
+        take(low, e, __shfl_xor_sync(0xFFFFFFFFu, k[e], j / RE), __shfl_xor_sync(0xFFFFFFFFu, ti[e], j / RE),
+             __shfl_xor_sync(0xFFFFFFFFu, v[e], j / RE));
+    }
+#pragma unroll
+    for (int jj = RE / 2; jj > 0; jj >>= 1) {
+      if (jj > j) continue;  // j: the first stride below RE of this stage
+#pragma unroll
+      for (int e = 0; e < RE; ++e)
+        if (!(e & jj)) {
+          const bool up = ((t * RE + e) & kk) == 0;
+          const int f = e | jj;
+          const bool sw = rank_less(k[f], ti[f], k[e], ti[e]) == up;
+          const uint64_t a = sw ? k[f] : k[e], b = sw ? k[e] : k[f];
+          const uint32_t ta = sw ? ti[f] : ti[e], tb = sw ? ti[e] : ti[f];
+          const uint32_t va = sw ? v[f] : v[e], vb = sw ? v[e] : v[f];
+          k[e] = a;
+          k[f] = b;
+          ti[e] = ta;
+          ti[f] = tb;
+          v[e] = va;
+          v[f] = vb;
+        }
+    }
+  }
+#pragma unroll
+  for (int e = 0; e < RE; ++e) {
+    const int64_t i = (int64_t)blockIdx.x * RTILE + t * RE + e;
+    out.key[i] = k[e];
+    out.tie[i] = ti[e];
+    out.val[i] = v[e];
+  }
+}
+
+// A thread per element.  The other tiles come through shared memory one after
+// another, the next one's loads in flight during the search of this one.
+__global__ __launch_bounds__(RT) void k_rank_place(RankArrays a, int64_t n, int tiles, uint64_t *keys, uint32_t *vals) {
+  __shared__ uint64_t sk[RTILE];
+  __shared__ uint32_t st[RTILE];
+  const int t = threadIdx.x;
+  const int64_t i = (int64_t)blockIdx.x * RT + t;  // RE blocks per tile
+  const int own = (int)(blockIdx.x / RE);
+  const uint64_t k = a.key[i];
+  const uint32_t ti = a.tie[i], v = a.val[i];
+  int64_t pos = i - (int64_t)own * RTILE;
+  uint64_t nk[RE];
+  uint32_t nt[RE];
+  auto fetch = [&](int x) {
+#pragma unroll
+    for (int e = 0; e < RE; ++e) {
+      nk[e] = a.key[(int64_t)x * RTILE + e * RT + t];
+      nt[e] = a.tie[(int64_t)x * RTILE + e * RT + t];
+    }
+  };
+  int x = own == 0 ? 1 : 0;
+  if (x < tiles) fetch(x);
+  while (x < tiles) {
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < RE; ++e) {
+      sk[e * RT + t] = nk[e];
+      st[e * RT + t] = nt[e];
+    }
+    __syncthreads();
+    const int next = x + 1 == own ? x + 2 : x + 1;
+    if (next < tiles) fetch(next);
+    const bool first = x < own;  // equal pairs of an earlier tile come first
+    int lo = 0;                  // elements of tile x before this one
+#pragma unroll
+    for (int s = RTILE / 2; s > 0; s >>= 1) {
+      const uint64_t kp = sk[lo + s - 1];
+      const uint32_t tp = st[lo + s - 1];
+      const bool before = first ? !rank_less(k, ti, kp, tp) : rank_less(kp, tp, k, ti);
+      lo += before ? s : 0;
+    }
+    lo += first ? !rank_less(k, ti, sk[lo], st[lo]) : rank_less(sk[lo], st[lo], k, ti);
+    pos += lo;
+    x = next;
+  }
+  if ((int64_t)v < n) {  // not padding
+    keys[pos] = k;
+    vals[pos] = v;
+  }
+}
+
+psi_status rank_sort(const EncodeSpec &enc, int64_t n, const uint32_t *tie_ids, uint64_t *keys, uint32_t *vals,
+                     int *d_status, cudaStream_t s) {
+  const int tiles = (int)ceil_div(n, RTILE);
+  const int64_t pad = (int64_t)tiles * RTILE;
+  Buf<uint64_t> scratch;
+  psi_status st = scratch.alloc(2 * pad, s);
+  if (st) return st;
+  RankArrays a{scratch.p, reinterpret_cast<uint32_t *>(scratch.p + pad), nullptr};
+  a.val = a.tie + pad;
+  if (enc.dim == 2 && enc.curve == CURVE_MORTON)
+    PSI_LAUNCH_NAMED("k_rank_tiles", (k_rank_tiles<2, 0>), tiles, RT, 0, s, enc, tie_ids, n, a, d_status);
+  else if (enc.dim == 2)
+    PSI_LAUNCH_NAMED("k_rank_tiles", (k_rank_tiles<2, 1>), tiles, RT, 0, s, enc, tie_ids, n, a, d_status);
+  else if (enc.curve == CURVE_MORTON)
+    PSI_LAUNCH_NAMED("k_rank_tiles", (k_rank_tiles<3, 0>), tiles, RT, 0, s, enc, tie_ids, n, a, d_status);
+  else
+    PSI_LAUNCH_NAMED("k_rank_tiles", (k_rank_tiles<3, 1>), tiles, RT, 0, s, enc, tie_ids, n, a, d_status);
+  PSI_LAUNCH(k_rank_place, (unsigned)(pad / RT), RT, 0, s, a, n, tiles, keys, vals);
+  PSI_CK(cudaGetLastError());
+  return PSI_OK;
+}
+
 }  // namespace
 
 // ---------------------------------------------------------------------------
@@ -1233,6 +1434,7 @@ psi_status sort_pairs(const EncodeSpec &enc, const uint64_t *keys_in, const uint
   if (encode && (enc.dim != 2 && enc.dim != 3)) return PSI_ERR_INVALID;
   key_bits = std::max(1, std::min(64, key_bits));
   psi_status st;
+  if (encode && n <= kRankSort && radix_bits == 0) return rank_sort(enc, n, tie_ids, kbuf0, vbuf0, d_status, s);
   switch (pick_radix(key_bits, radix_bits)) {
     case 10:
       st = sort_pairs_rb<10>(enc, keys_in, vals_in, n, key_bits, kbuf0, vbuf0, kbuf1, vbuf1, d_status, s, out, false);
