@@ -108,17 +108,17 @@ __global__ void k_insert_plan(const int32_t *cnt, const int32_t *sbeg, const int
 
 constexpr int MAXPL = 4;  // points per lane in one block (C <= 128)
 
-// Sorts, in place by (key, id), the cnt (<= MAXPL * 32) points of one leaf
-// block starting at slot s0: the whole warp ranks every point against all
-// others and writes it to its rank.
-template <int D>
+// Sorts, in place by (key, id), the cnt (<= R * 32) points of one leaf block
+// starting at slot s0: the whole warp ranks every point against all others and
+// writes it to its rank.
+template <int D, int R>
 __device__ __forceinline__ void sort_leaf_block(Pool &pool, uint32_t s0, int cnt) {
   const int lane = threadIdx.x & 31;
-  uint64_t k[MAXPL];
-  uint32_t id[MAXPL];
-  int32_t c[MAXPL][D];
+  uint64_t k[R];
+  uint32_t id[R];
+  int32_t c[R][D];
 #pragma unroll
-  for (int r = 0; r < MAXPL; ++r) {
+  for (int r = 0; r < R; ++r) {
     const int e = r * 32 + lane;
     k[r] = ~0ull;
     id[r] = 0xFFFFFFFFu;
@@ -129,20 +129,20 @@ __device__ __forceinline__ void sort_leaf_block(Pool &pool, uint32_t s0, int cnt
       for (int d = 0; d < D; ++d) c[r][d] = pool.px[d][s0 + e];
     }
   }
-  int rank[MAXPL] = {0, 0, 0, 0};
-  for (int r2 = 0; r2 < MAXPL; ++r2) {
+  int rank[R] = {};
+  for (int r2 = 0; r2 < R; ++r2) {
     if (r2 * 32 >= cnt) break;
     for (int sl = 0; sl < 32; ++sl) {
       const uint64_t kf = __shfl_sync(0xFFFFFFFFu, k[r2], sl);
       const uint32_t idf = __shfl_sync(0xFFFFFFFFu, id[r2], sl);
       if (r2 * 32 + sl >= cnt) break;
 #pragma unroll
-      for (int r = 0; r < MAXPL; ++r) rank[r] += kid_less(kf, idf, k[r], id[r]);
+      for (int r = 0; r < R; ++r) rank[r] += kid_less(kf, idf, k[r], id[r]);
     }
   }
   __syncwarp();
 #pragma unroll
-  for (int r = 0; r < MAXPL; ++r) {
+  for (int r = 0; r < R; ++r) {
     const int e = r * 32 + lane;
     if (e < cnt) {
       pool.pkey[s0 + rank[r]] = k[r];
@@ -157,7 +157,7 @@ __device__ __forceinline__ void sort_leaf_block(Pool &pool, uint32_t s0, int cnt
 // Sorts, in place, the block of every leaf that will be re-wrapped.  A warp
 // takes 32 leaves: one lane per leaf finds the few that overflow, then the
 // warp sorts each of those.
-template <int D>
+template <int D, int R>
 __global__ void k_sort_overflow_leaves(const int32_t *ncnt, const uint32_t *nref, const int32_t *sbeg,
                                        const int32_t *send, int64_t L, int C, Pool pool, int lpw) {
   const int lane = threadIdx.x & 31;
@@ -168,7 +168,7 @@ __global__ void k_sort_overflow_leaves(const int32_t *ncnt, const uint32_t *nref
     while (todo) {
       const int64_t j = j0 + __ffs(todo) - 1;
       todo &= todo - 1;
-      sort_leaf_block<D>(pool, nref[j], ncnt[j]);
+      sort_leaf_block<D, R>(pool, nref[j], ncnt[j]);
     }
   }
 }
@@ -644,7 +644,7 @@ __global__ void k_wrap_plan(const int32_t *cnt, const int32_t *start, const int6
 
 // Sorts, in place, the block of every leaf of a group (a group's points in
 // leaf order are then sorted by (key, id) as a whole).
-template <int D>
+template <int D, int R>
 __global__ void k_sort_flagged_leaves(const int32_t *cnt, const uint32_t *ref, const int32_t *flag, int64_t L,
                                       Pool pool, int lpw) {
   const int lane = threadIdx.x & 31;
@@ -655,7 +655,7 @@ __global__ void k_sort_flagged_leaves(const int32_t *cnt, const uint32_t *ref, c
     while (todo) {
       const int64_t j = j0 + __ffs(todo) - 1;
       todo &= todo - 1;
-      sort_leaf_block<D>(pool, ref[j], cnt[j]);
+      sort_leaf_block<D, R>(pool, ref[j], cnt[j]);
     }
   }
 }
@@ -856,12 +856,17 @@ psi_status spac_insert(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
 
   const int64_t base_block = ix->pool_used;
   if ((st = grow_pool(ix, (base_block + NB) * ix->C, base_block * ix->C, s))) return st;
-  if (ix->D == 2)
-    PSI_LAUNCH_NAMED("k_sort_overflow_leaves", k_sort_overflow_leaves<2>, warp_grid(ceil_div(L, lpw)), 256, 0, s,
-                     ix->nodes.cnt, ix->nodes.ref, sbeg.p, send.p, L, ix->C, ix->pool, lpw);
-  else
-    PSI_LAUNCH_NAMED("k_sort_overflow_leaves", k_sort_overflow_leaves<3>, warp_grid(ceil_div(L, lpw)), 256, 0, s,
-                     ix->nodes.cnt, ix->nodes.ref, sbeg.p, send.p, L, ix->C, ix->pool, lpw);
+#define SORT_LEAVES(DD, RR)                                                                                    \
+  PSI_LAUNCH_NAMED("k_sort_overflow_leaves", (k_sort_overflow_leaves<DD, RR>), warp_grid(ceil_div(L, lpw)), 256, 0, s, ix->nodes.cnt, ix->nodes.ref, sbeg.p, \
+                   send.p, L, ix->C, ix->pool, lpw)
+  if (ix->D == 2) {
+    if (ix->C <= 64) SORT_LEAVES(2, 2);
+    else SORT_LEAVES(2, MAXPL);
+  } else {
+    if (ix->C <= 64) SORT_LEAVES(3, 2);
+    else SORT_LEAVES(3, MAXPL);
+  }
+#undef SORT_LEAVES
 
   NodeArrays na;
   uint64_t *nsk = nullptr;
@@ -995,12 +1000,17 @@ psi_status spac_delete(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
   const int64_t Lnew = h3[0], NB = h3[1];
   const int64_t base_block = ix->pool_used;
   if ((st = grow_pool(ix, (base_block + NB) * ix->C, base_block * ix->C, s))) return st;
-  if (ix->D == 2)
-    PSI_LAUNCH_NAMED("k_sort_flagged_leaves", k_sort_flagged_leaves<2>, warp_grid(ceil_div(L, lpw)), 256, 0, s,
-                     ix->nodes.cnt, ix->nodes.ref, ingroup.p, L, ix->pool, lpw);
-  else
-    PSI_LAUNCH_NAMED("k_sort_flagged_leaves", k_sort_flagged_leaves<3>, warp_grid(ceil_div(L, lpw)), 256, 0, s,
-                     ix->nodes.cnt, ix->nodes.ref, ingroup.p, L, ix->pool, lpw);
+#define SORT_LEAVES(DD, RR)                                                                                    \
+  PSI_LAUNCH_NAMED("k_sort_flagged_leaves", (k_sort_flagged_leaves<DD, RR>), warp_grid(ceil_div(L, lpw)), 256, 0, s, ix->nodes.cnt, ix->nodes.ref, ingroup.p, \
+                   L, ix->pool, lpw)
+  if (ix->D == 2) {
+    if (ix->C <= 64) SORT_LEAVES(2, 2);
+    else SORT_LEAVES(2, MAXPL);
+  } else {
+    if (ix->C <= 64) SORT_LEAVES(3, 2);
+    else SORT_LEAVES(3, MAXPL);
+  }
+#undef SORT_LEAVES
   NodeArrays na;
   uint64_t *nsk = nullptr;
   uint32_t *nsi = nullptr;
