@@ -454,8 +454,8 @@ __global__ __launch_bounds__(BT) void k_batch_build(BuildArgs a) {
 // finish.  Such a batch is sorted as a whole: by the low 8 key bits first, then
 // by (index number, the other key bits) in one word, with the device's digit
 // passes; the leaves of all indexes are then gathered at once.  The layout is
-// the same.  256 indexes of 1e3 to 1e6 points (3.7e7 in all), build: 19.3 ms by
-// blocks, 5.0 ms device-wide; 4096 of them (5.95e8) take 67 ms by blocks.
+// the same.  256 indexes of 1e3 to 1e6 points (3.7e7 in all), build kernels: 19.2 ms
+// by blocks, 4.5 ms device-wide; 4096 of them (5.95e8) take 67 ms by blocks.
 
 // Index that position p of the concatenated arrays belongs to.
 __device__ __forceinline__ int segment_of(const int64_t *off, int nidx, int64_t p) {

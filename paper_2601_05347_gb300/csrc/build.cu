@@ -278,8 +278,8 @@ __global__ void k_summarise(NodeW nodes, int64_t child_off, int64_t child_n, int
 
 // All remaining levels, from one of at most kTopParents parents up, by one
 // block: a launch of its own costs a small level more than its work.  Under the
-// event timer, 625 leaves (20 and 1 parents): two launches 11.3 us, one 6.4; 3e5
-// leaves (9766, 306, 10, 1): four 23.6 us, two 20.6.
+// event timer, 625 leaves (20 and 1 parents): two launches 11.0 us, one 6.4; 3e5
+// leaves (9766, 306, 10, 1): four 23.6 us, two 20.8.
 constexpr int kTopParents = 384;
 
 template <int D>

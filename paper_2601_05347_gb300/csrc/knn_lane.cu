@@ -25,9 +25,8 @@
 // against 1190 for two queries per warp, issue slots 55 % busy, 26 of 64 warps
 // resident, L1 hits 64 %, DRAM 7 %).  Blocks of 128 threads at 64 to 80
 // registers: at 72 to 96 registers there were no spills, but fewer warps, and
-// 3D 10-NN took 5 to 8 % longer.  Queries that scan their own queue of leaves
-// (no shared pool) kept 40 to 50 % of the lanes busy and took 30 % longer; an
-// exact (distance, id) list kept during the search, twice as long.
+// 3D SPaC-H 10-NN took 7 to 8 % longer.  The pool is shared by the warp because queries that
+// scan their own queues of leaves leave lanes idle when the lengths differ.
 // 1e7 10-NN on 1e8 2D Varden points, whole call: 18.9 -> 8.2 ms.
 //
 // Exactness is k_knn's: exact int64 distances, ties by id, a child or leaf

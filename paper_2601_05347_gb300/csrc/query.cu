@@ -1021,8 +1021,8 @@ __device__ __forceinline__ void seg_sort(uint32_t *ids, int len, uint32_t *sm) {
 // per thread keep most of the network in registers: at 1024 ids, 15 of its 55
 // stages are shuffles (whose rate bounds it) with 32 values per thread, 30
 // with 8.  The classes are listed first and every warp or block takes the next
-// segment of its list: taken in strides over all segments, some found twice as
-// many of their class as others (890 us against 740).  5e4 boxes of 1259 ids on
+// segment of its list: taken in strides over all segments, some find more
+// of their class than others.  5e4 boxes of 1259 ids on
 // average (6.3e7 ids): 590 us, against 6.1 ms for one 1024-thread block per
 // segment with a network in shared memory and a barrier per stage; bound by
 // instruction issue (about 110 per id and 32 lanes).

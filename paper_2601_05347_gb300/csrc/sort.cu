@@ -1160,8 +1160,8 @@ static psi_status launch_hist_as(const uint64_t *kin, const EncodeSpec &enc, int
   return PSI_OK;
 }
 
-// Building the larger Hilbert tables takes a block about 2 us, as long as a
-// small sort's whole count.
+// Building the larger Hilbert tables is work per block that a small sort's few
+// keys do not pay back.
 constexpr int64_t kBigTables = int64_t(1) << 18;
 
 template <int MODE, int D, int CURVE, int RB>
@@ -1534,7 +1534,8 @@ __global__ void k_scan_sums(int64_t *sums, int64_t nb, int64_t *total) {
 // How the apply kernels get their block's offset: from the scanned block sums
 // (k_scan_sums), or, up to kScanDirect blocks, by adding up the sums before it
 // themselves (16 KB of L2 reads at most), which spares the launch between the
-// other two: 3 us of the 9 that a scan of 1e6 elements took.
+// other two: 6.1 of 18.8 us per scan under the event timer (24 scans of a float
+// build of 3e6 points).
 constexpr int64_t kScanDirect = 2048;
 
 // Offset of this block; DIRECT: the last block writes the grand total.  Call

@@ -32,7 +32,7 @@ namespace {
 // Leaves a warp of the leaf kernels takes: 32 (one lane per leaf finds the
 // touched ones, the warp then works on each) where that leaves enough warps to
 // fill the chip, else fewer, for the warp works through its touched leaves one
-// after another (625 leaves, all touched: delete 57 -> 13 us).
+// after another (625 leaves, all touched: delete 57.3 -> 8.0 us).
 int leaves_per_warp(int64_t L) {
   int w = 32;
   while (w > 1 && ceil_div(L, w) < (int64_t)num_sms() * 48) w /= 2;
