@@ -237,7 +237,8 @@ def source_digest(files) -> str:
 
 
 KERNEL_SOURCES = {"k_knn": ["paper_2601_05347_gb300/csrc/query.cu", "paper_2601_05347_gb300/csrc/klist.cuh",
-                            "paper_2601_05347_gb300/csrc/index.cuh"]}
+                            "paper_2601_05347_gb300/csrc/index.cuh", "paper_2601_05347_gb300/csrc/knn_lane.cu",
+                            "paper_2601_05347_gb300/csrc/knn.cuh"]}
 
 
 def profiled_traffic(kernel: str, workload_name: str):

@@ -21,9 +21,9 @@
 // the notes are put in exact (distance, id) order by a sorting network.
 //
 // What bounds it: instruction issue and the latency of the scattered loads
-// (ncu, 1e6 10-NN on 1e7 2D Varden points: 436 warp instructions per query
+// (ncu, 1e6 10-NN on 1e7 2D Varden points: 456 warp instructions per query
 // against 1190 for two queries per warp, issue slots 55 % busy, 26 of 64 warps
-// resident, L1 hits 64 %, DRAM 7 %).  Blocks of 128 threads at 64 to 80
+// resident, L1 hits 65 %, DRAM 7 %).  Blocks of 128 threads at 64 to 80
 // registers: at 72 to 96 registers there were no spills, but fewer warps, and
 // 3D SPaC-H 10-NN took 7 to 8 % longer.  The pool is shared by the warp because queries that
 // scan their own queues of leaves leave lanes idle when the lengths differ.
