@@ -30,6 +30,7 @@ struct psi_batch {
   int rb = 8;  // digit width of the block sort
   int seg_bits = 0;   // bits of an index number
   bool wide = false;  // built by device-wide sorts (few large indexes) instead of a block each
+  uint32_t *sort_scratch = nullptr;  // of those sorts (wide only)
   int nidx = 0;
   int64_t total = 0;
   std::vector<int64_t> off, leaves, node_off, block_off, nodes_per;
@@ -642,12 +643,15 @@ psi_status build_wide(psi_batch *b, const BuildArgs &a, cudaStream_t s) {
   SortResult r;
   EncodeSpec none;
   PSI_LAUNCH_NAMED("k_wide_keys", (k_wide_keys<D, CURVE>), grid(n), 256, 0, s, a.pts, n, a.bits, b->kA, b->vA, a.status);
-  if ((st = sort_pairs(none, b->kA, b->vA, n, 8, nullptr, b->kB, b->vB, b->kA, b->vA, a.status, s, &r))) return st;
+  if ((st = sort_pairs(none, b->kA, b->vA, n, 8, nullptr, b->kB, b->vB, b->kA, b->vA, a.status, s, &r, 0,
+                       b->sort_scratch)))
+    return st;
   const int low = std::max(b->key_bits - 8, 0);
   PSI_LAUNCH(k_wide_segment, grid(n), 256, 0, s, b->d_off, b->nidx, low, r.vals, n, r.keys);
   uint64_t *k0 = r.keys == b->kA ? b->kB : b->kA;
   uint32_t *v0 = r.vals == b->vA ? b->vB : b->vA;
-  if ((st = sort_pairs(none, r.keys, r.vals, n, low + b->seg_bits, nullptr, k0, v0, r.keys, r.vals, a.status, s, &r)))
+  if ((st = sort_pairs(none, r.keys, r.vals, n, low + b->seg_bits, nullptr, k0, v0, r.keys, r.vals, a.status, s, &r,
+                       0, b->sort_scratch)))
     return st;
   PSI_LAUNCH_NAMED("k_wide_full", (k_wide_full<D, CURVE>), grid(n), 256, 0, s, a.pts, r.vals, n, a.bits, r.keys);
   // the sort's free key buffer lists the long runs (8 bytes per 33 positions)
@@ -722,7 +726,8 @@ static void batch_free(psi_batch *b) {
   for (void *p : {(void *)b->d_off, (void *)b->d_block_off, (void *)b->d_node_off, (void *)b->d_order,
                   (void *)b->d_root, (void *)b->d_queue, (void *)b->d_status, (void *)b->kA, (void *)b->kB,
                   (void *)b->vA, (void *)b->vB, (void *)b->d_qroot, (void *)b->d_qseg, (void *)b->d_qoff,
-                  (void *)b->qk0, (void *)b->qk1, (void *)b->qv0, (void *)b->qv1, (void *)b->d_nhard})
+                  (void *)b->qk0, (void *)b->qk1, (void *)b->qv0, (void *)b->qv1, (void *)b->d_nhard,
+                  (void *)b->sort_scratch})
     DevMem::free(p, s);
   delete b;
 }
@@ -834,6 +839,9 @@ psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int
     if ((st = DevMem::alloc((void **)&b->kB, sizeof(uint64_t) * N, s))) break;
     if ((st = DevMem::alloc((void **)&b->vA, sizeof(uint32_t) * N, s))) break;
     if ((st = DevMem::alloc((void **)&b->vB, sizeof(uint32_t) * N, s))) break;
+    if (b->wide &&
+        (st = DevMem::alloc((void **)&b->sort_scratch, sizeof(uint32_t) * sort_scratch_words(b->total), s)))
+      break;
     cudaError_t e;
     if ((e = cudaMemcpyAsync(b->d_off, b->off.data(), sizeof(int64_t) * (nidx + 1), cudaMemcpyHostToDevice, s)) ||
         (e = cudaMemcpyAsync(b->d_block_off, b->block_off.data(), sizeof(int64_t) * (nidx + 1),

@@ -158,10 +158,15 @@ struct SortResult {
 // pairs (keys_in, vals_in) are sorted.  key_bits limits the digits sorted.
 // When tie_ids is non-null, runs of equal keys are re-ordered so that
 // tie_ids[value] increases (values are positions into tie_ids).
-// The result lives in one of the two caller-provided buffer pairs.
+// The result lives in one of the two caller-provided buffer pairs.  With
+// `scratch` (sort_scratch_words of n or more words), a sort of pairs by 8-bit
+// digits without tie_ids allocates nothing.
 psi_status sort_pairs(const EncodeSpec &enc, const uint64_t *keys_in, const uint32_t *vals_in, int64_t n,
                       int key_bits, const uint32_t *tie_ids, uint64_t *kbuf0, uint32_t *vbuf0, uint64_t *kbuf1,
-                      uint32_t *vbuf1, int *d_status, cudaStream_t s, SortResult *out, int radix_bits = 0);
+                      uint32_t *vbuf1, int *d_status, cudaStream_t s, SortResult *out, int radix_bits = 0,
+                      uint32_t *scratch = nullptr);
+// 32-bit words of scratch that are enough for any such sort of at most n pairs.
+size_t sort_scratch_words(int64_t n);
 
 // Device-wide exclusive scan of int64 values (out may alias in); writes the
 // grand total to d_total if non-null.

@@ -1232,7 +1232,8 @@ static int pick_radix(int /*key_bits*/, int requested) {
 template <int RB>
 static psi_status sort_pairs_rb(const EncodeSpec &enc, const uint64_t *keys_in, const uint32_t *vals_in, int64_t n,
                                 int key_bits, uint64_t *kbuf0, uint32_t *vbuf0, uint64_t *kbuf1, uint32_t *vbuf1,
-                                int *d_status, cudaStream_t s, SortResult *out, bool may_prefix) {
+                                int *d_status, cudaStream_t s, SortResult *out, bool may_prefix,
+                                uint32_t *given = nullptr) {
   using R = Radix<RB>;
   const bool encode = enc.pts != nullptr;
   const int passes_full = (key_bits + RB - 1) / RB;
@@ -1259,14 +1260,15 @@ static psi_status sort_pairs_rb(const EncodeSpec &enc, const uint64_t *keys_in, 
   psi_status st;
   // digit counts: a section per pass, then the prefix sort's first digit;
   // two look-back tables used alternately: pass p clears the table of pass p+1
-  // (one allocation: counts, tile counters, the two tables; all but the second
-  // table start at zero)
+  // (one allocation, or the caller's sort_scratch_words: counts, tile counters,
+  // the two tables; all but the second table start at zero)
   const size_t n_hist = (size_t)(passes_full + 1) * R::RADIX, n_look = (size_t)tiles * R::RADIX;
-  if ((st = scratch.alloc(n_hist + R::RADIX + 2 * n_look, s))) return st;
+  if (!given && (st = scratch.alloc(n_hist + R::RADIX + 2 * n_look, s))) return st;
+  uint32_t *const base = given ? given : scratch.p;
   struct {
     uint32_t *p;
-  } hist{scratch.p}, ctr{scratch.p + n_hist}, lookback{scratch.p + n_hist + R::RADIX};
-  PSI_CK(cudaMemsetAsync(scratch.p, 0, sizeof(uint32_t) * (n_hist + R::RADIX + n_look), s));
+  } hist{base}, ctr{base + n_hist}, lookback{base + n_hist + R::RADIX};
+  PSI_CK(cudaMemsetAsync(base, 0, sizeof(uint32_t) * (n_hist + R::RADIX + n_look), s));
 
   // Hilbert keys cost more arithmetic than their 8-byte write and read: the
   // histogram pass computes them once and writes them out; the first digit
@@ -1420,9 +1422,17 @@ static psi_status sort_pairs_rb(const EncodeSpec &enc, const uint64_t *keys_in, 
   return PSI_OK;
 }
 
+size_t sort_scratch_words(int64_t n) {
+  constexpr size_t RADIX = Radix<8>::RADIX;
+  // small sorts take smaller tiles: the most tiles may not be the largest sort's
+  const int64_t tiles = std::max(ceil_div(n, TILE), ceil_div(std::min(n, kSmallSort), (int64_t)ST * SI_SMALL));
+  return (MAX_PASSES + 2) * RADIX + 2 * (size_t)tiles * RADIX;
+}
+
 psi_status sort_pairs(const EncodeSpec &enc, const uint64_t *keys_in, const uint32_t *vals_in, int64_t n,
                       int key_bits, const uint32_t *tie_ids, uint64_t *kbuf0, uint32_t *vbuf0, uint64_t *kbuf1,
-                      uint32_t *vbuf1, int *d_status, cudaStream_t s, SortResult *out, int radix_bits) {
+                      uint32_t *vbuf1, int *d_status, cudaStream_t s, SortResult *out, int radix_bits,
+                      uint32_t *scratch) {
   out->keys = kbuf0;
   out->vals = vbuf0;
   if (n <= 0) return PSI_OK;
@@ -1444,7 +1454,7 @@ psi_status sort_pairs(const EncodeSpec &enc, const uint64_t *keys_in, const uint
       break;
     default:
       st = sort_pairs_rb<8>(enc, keys_in, vals_in, n, key_bits, kbuf0, vbuf0, kbuf1, vbuf1, d_status, s, out,
-                            tie_ids != nullptr);
+                            tie_ids != nullptr, scratch);
   }
   if (st) return st;
 
