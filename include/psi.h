@@ -164,6 +164,9 @@ typedef struct psi_batch psi_batch;
 psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int32_t nidx, int32_t threads,
                             void *stream, psi_batch **out);
 
+/* 1 where psi_batch_create with these (valid) arguments chooses device-wide sorts. */
+int32_t psi_batch_device_wide(const psi_config *cfg, const int64_t *h_offsets, int32_t nidx, int32_t threads);
+
 /* Builds every index of the batch (Algorithm 3 per index: curve keys, (key, id)
  * sort, leaf wrapping, summaries) in ONE persistent kernel launch: each thread
  * block takes whole indexes, largest first, from an atomic queue (or, see

@@ -732,6 +732,30 @@ static void batch_free(psi_batch *b) {
   delete b;
 }
 
+// Bits of an index number beside the key.
+static int segment_bits(int32_t nidx) {
+  int bits = 0;
+  while ((int64_t(1) << bits) < nidx) ++bits;
+  return bits;
+}
+
+// Built by device-wide sorts: where the caller left the block's form open, the
+// sorts take the batch (kSortLimit, and index numbers fit beside the keys), and
+// the largest index, or an even share of the points, keeps a block busy 1.3
+// times as long as they take.  A block takes as long for a point as a digit
+// pass of the whole batch for kBlockPoint of its points (18 ns, 0.013 ns); the
+// gathers count as two passes, and the launches as kWideStart of a block's points.
+static bool device_wide(const psi_config *cfg, const int64_t *off, int32_t nidx, int32_t threads) {
+  constexpr double kBlockPoint = 1385, kWideStart = 11100;
+  const int64_t total = off[nidx];
+  const int word = std::max(cfg->dim * cfg->coord_bits - 8, 0) + segment_bits(nidx);
+  if (threads != 0 || cfg->radix_bits != 0 || total >= kSortLimit || word > 64) return false;
+  int64_t longest = total / num_sms();
+  for (int32_t i = 0; i < nidx; ++i) longest = std::max(longest, off[i + 1] - off[i]);
+  const double passes = 1 + ceil_div(word, 8) + 2;
+  return (double)longest > 1.3 * (passes * (double)total / kBlockPoint + kWideStart);
+}
+
 extern "C" {
 
 psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int32_t nidx, int32_t threads,
@@ -806,17 +830,8 @@ psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int
     set_error("batch too large for 32-bit node and slot references");
     return PSI_ERR_INVALID;
   }
-  // Device-wide, where the caller left the block's form open, when the largest index, or an even share of the points, keeps a
-  // block busy 1.3 times as long as the digit passes of the whole batch take
-  // (18 ns per point in a block; 0.013 ns per point and pass, and two passes'
-  // worth of gathers), and index numbers fit beside the keys.
-  while ((int64_t(1) << b->seg_bits) < nidx) ++b->seg_bits;
-  int64_t largest = 0;
-  for (int i = 0; i < nidx; ++i) largest = std::max(largest, b->off[i + 1] - b->off[i]);
-  const double passes = 1 + ceil_div(std::max(b->key_bits - 8, 0) + b->seg_bits, 8) + 2;
-  const double by_block = 18e-9 * (double)std::max<int64_t>(largest, b->total / num_sms());
-  b->wide = threads == 0 && cfg->radix_bits == 0 && b->total < (int64_t(1) << 30) && std::max(b->key_bits - 8, 0) + b->seg_bits <= 64 &&
-            by_block > 1.3 * (0.013e-9 * passes * (double)b->total + 200e-6);
+  b->seg_bits = segment_bits(nidx);
+  b->wide = device_wide(cfg, h_offsets, nidx, threads);
   std::vector<int32_t> order(nidx);
   std::iota(order.begin(), order.end(), 0);
   std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
@@ -861,6 +876,10 @@ psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int
   }
   *out = b;
   return PSI_OK;
+}
+
+int32_t psi_batch_device_wide(const psi_config *cfg, const int64_t *h_offsets, int32_t nidx, int32_t threads) {
+  return cfg && h_offsets && nidx >= 1 && device_wide(cfg, h_offsets, nidx, threads) ? 1 : 0;
 }
 
 psi_status psi_batch_build(psi_batch *b, const int32_t *d_pts, const uint32_t *d_ids, void *stream) {

@@ -153,6 +153,9 @@ struct SortResult {
   int local = -1;
 };
 
+// A sort takes fewer pairs than this: a look-back word counts in 30 bits.
+constexpr int64_t kSortLimit = (int64_t(1) << 30) - 1;
+
 // Sorts n pairs.  If enc.pts is non-null the keys are computed from the points
 // on first touch and the values are the input positions 0..n-1; otherwise the
 // pairs (keys_in, vals_in) are sorted.  key_bits limits the digits sorted.

@@ -54,6 +54,7 @@ constexpr int SW = ST / 32;
 constexpr int MAX_PASSES = 8;  // 64-bit keys at 8-bit digits
 
 constexpr uint32_t LB_AGG = 1u << 30, LB_PRE = 2u << 30, LB_VAL = (1u << 30) - 1;
+static_assert(LB_VAL == kSortLimit, "a look-back word holds a count below kSortLimit");
 // Predecessor tiles read per look-back step.  More read L2 faster than they save
 // steps in a large sort (1e8 pairs: 8 tiles 0.861 ms, 16 0.931); a small one's
 // chain is short and the words are all there.
@@ -1436,8 +1437,8 @@ psi_status sort_pairs(const EncodeSpec &enc, const uint64_t *keys_in, const uint
   out->keys = kbuf0;
   out->vals = vbuf0;
   if (n <= 0) return PSI_OK;
-  if (n >= (int64_t)LB_VAL) {
-    set_error("sort: more than 2^30-1 pairs in one sort");
+  if (n >= kSortLimit) {
+    set_error("sort: 2^30-1 or more pairs in one sort");
     return PSI_ERR_INVALID;
   }
   const bool encode = enc.pts != nullptr;
@@ -1945,7 +1946,7 @@ extern "C" psi_status psi_test_sort_withheld_tile(uint64_t *d_keys, uint32_t *d_
                                                   int64_t withheld_tile, uint32_t spin_limit, void *stream) {
   using namespace psi;
   set_error("");
-  if (n < 0 || (n > 0 && (!d_keys || !d_vals)) || n >= (int64_t)LB_VAL || spin_limit < 1) {
+  if (n < 0 || (n > 0 && (!d_keys || !d_vals)) || n >= kSortLimit || spin_limit < 1) {
     set_error("invalid test sort arguments");
     return PSI_ERR_INVALID;
   }

@@ -72,6 +72,7 @@ def lib():
             "psi_sort_pairs_noalloc": (st, [P, P, i64, i32, P]),
             "psi_test_sort_withheld_tile": (st, [P, P, i64, i64, ctypes.c_uint32, P]),
             "psi_batch_create": (st, [P, P, i32, i32, P, P]),
+            "psi_batch_device_wide": (i32, [P, P, i32, i32]),
             "psi_batch_build": (st, [P, P, P, P]),
             "psi_batch_knn_reserve": (st, [P, i64, P]),
             "psi_batch_knn": (st, [P, P, P, i64, i32, P, P, P]),
@@ -355,6 +356,17 @@ class Batch:
             self.close()
         except Exception:
             pass
+
+
+def batch_device_wide(offsets, *, dim: int = 2, kind: int | str = SPAC_H, leaf_size: int = 32,
+                      coord_bits: int | None = None, threads: int = 0, radix_bits: int = 0) -> bool:
+    """Whether a Batch of these arguments is built by device-wide sorts instead of a block per index."""
+    import numpy as np
+    cfg = Config(dim, KINDS[kind] if isinstance(kind, str) else kind, leaf_size,
+                 coord_bits or (30 if dim == 2 else 21), 32, radix_bits)
+    off = np.ascontiguousarray(offsets, dtype=np.int64)
+    return bool(lib().psi_batch_device_wide(ctypes.byref(cfg), off.ctypes.data_as(ctypes.c_void_p), len(off) - 1,
+                                            threads))
 
 
 class FConfig(ctypes.Structure):
