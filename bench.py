@@ -587,7 +587,7 @@ def run_batched(nidx: int, steps: int, warmup: int, rank: int = 0, max_size: int
     t_off, t_qoff = off[: ns + 1], qoff[: ns + 1]
     phi, threads, rbits, tinfo = tune.autotune(t_off, dp[: t_off[-1]], di[: t_off[-1]], dq[: t_qoff[-1]],
                                                dqo[: ns + 1], int(t_qoff[-1]), k, dim=2, kind="spac_h",
-                                               dist="half-uniform-half-varden", sizes=sizes[:ns])
+                                               dist="half-uniform-half-varden", sizes=sizes[:ns], batch_off=off)
     b = psi.Batch(off, kind="spac_h", leaf_size=phi, threads=threads, radix_bits=rbits)
     b.reserve(nq)
     oi = torch.empty((nq, k), dtype=torch.int32, device=dev)

@@ -4,8 +4,11 @@ Chooses the leaf size (16, 32, 64), the thread-block size of the persistent
 build (256, 512, 1024) and the digit width of its block sort (8 or 11 bits;
 11-bit digits with 256 or 512 threads only) by timing build + k-NN on a sample
 of the batch with CUDA events, and caches the choice in a JSON file keyed by
-(kind, dim, size bucket, distribution).  Results do not depend on the choice:
-k-NN answers are defined by the point set alone.
+(kind, dim, size bucket, distribution).  Where the whole batch is one that the
+library builds by device-wide sorts when the block's form is left open (threads
+and digit width 0), that form is timed too, and the choice is kept under a key
+of its own.  Results do not depend on the choice: k-NN answers are defined by
+the point set alone.
 """
 from __future__ import annotations
 
@@ -66,9 +69,17 @@ def time_config(off, dpts, dids, dq, dqoff, nq, k, *, dim, kind, leaf_size, thre
     return e0.elapsed_time(e1) / reps
 
 
-def autotune(off, dpts, dids, dq, dqoff, nq, k, *, dim: int, kind: str, dist: str, sizes, refresh=False):
-    """Best (leaf_size, threads, radix_bits) for this batch shape, from the cache or by timing."""
+def autotune(off, dpts, dids, dq, dqoff, nq, k, *, dim: int, kind: str, dist: str, sizes, refresh=False,
+             batch_off=None):
+    """Best (leaf_size, threads, radix_bits) for this batch shape, from the cache or by timing.
+
+    off: offsets of the timed sample; batch_off: those of the whole batch, where that is larger."""
     key = cache_key(kind, dim, np.asarray(sizes), dist)
+    whole = off if batch_off is None else batch_off
+    # the sample must take the form too: its time is what is compared
+    wide = off is not None and all(psi.batch_device_wide(o, dim=dim, kind=kind) for o in (off, whole))
+    if wide:
+        key += "/wide"
     cache = _load()
     if key in cache and not refresh and "radix_bits" in cache[key]:
         return cache[key]["leaf_size"], cache[key]["threads"], cache[key]["radix_bits"], cache[key]
@@ -80,6 +91,9 @@ def autotune(off, dpts, dids, dq, dqoff, nq, k, *, dim: int, kind: str, dist: st
                     continue  # 11-bit digits do not fit a 1024-thread block's shared memory
                 trials[f"{phi}/{th}/{rb}"] = time_config(off, dpts, dids, dq, dqoff, nq, k, dim=dim, kind=kind,
                                                          leaf_size=phi, threads=th, radix_bits=rb)
+        if wide:
+            trials[f"{phi}/0/0"] = time_config(off, dpts, dids, dq, dqoff, nq, k, dim=dim, kind=kind, leaf_size=phi,
+                                               threads=0, radix_bits=0)
     best = min(trials, key=trials.get)
     phi, th, rb = (int(x) for x in best.split("/"))
     cache[key] = {"leaf_size": phi, "threads": th, "radix_bits": rb, "ms": trials[best], "trials_ms": trials}
