@@ -1017,17 +1017,17 @@ __device__ __forceinline__ void seg_sort(uint32_t *ids, int len, uint32_t *sm) {
 }
 
 // The segments by length, each class sorted by a kernel of its own: a warp per
-// segment up to 1024 ids, then blocks of 64, 128 and 512 threads.  Many values
-// per thread keep most of the network in registers: at 1024 ids, 15 of its 55
-// stages are shuffles (whose rate bounds it) with 32 values per thread, 30
-// with 8.  The classes are listed first and every warp or block takes the next
+// segment up to 1024 ids, then blocks of 64, 128 and 512 threads, then
+// k_sort_seg_any.  Many values per thread keep most of the network in registers:
+// at 1024 ids, 15 of its 55 stages are shuffles (whose rate bounds it) with 32
+// values per thread; 28 are between threads with 8.  The classes are listed first and every warp or block takes the next
 // segment of its list: taken in strides over all segments, some find more
 // of their class than others.  5e4 boxes of 1259 ids on
 // average (6.3e7 ids): 590 us, against 6.1 ms for one 1024-thread block per
 // segment with a network in shared memory and a barrier per stage; bound by
 // instruction issue (about 110 per id and 32 lanes).
-constexpr int kSegClasses = 4;
-constexpr int kSeg0 = 1024, kSeg1 = 2048, kSeg2 = 4096;  // largest of classes 0 to 2
+constexpr int kSegClasses = 5;
+constexpr int kSeg0 = 1024, kSeg1 = 2048, kSeg2 = 4096, kSeg3 = 16384;  // largest of classes 0 to 3
 
 struct SegLists {
   uint32_t *list;  // [kSegClasses][nq]
@@ -1040,7 +1040,7 @@ __global__ __launch_bounds__(256) void k_seg_classes(const int64_t *offsets, Seg
   const int64_t rounds = (l.nq + 31) / 32 * 32;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < rounds; q += (int64_t)gridDim.x * blockDim.x) {
     const int64_t len = q < l.nq ? offsets[q + 1] - offsets[q] : 0;
-    const int c = len < 2 ? -1 : (len > kSeg0) + (len > kSeg1) + (len > kSeg2);
+    const int c = len < 2 ? -1 : (len > kSeg0) + (len > kSeg1) + (len > kSeg2) + (len > kSeg3);
 #pragma unroll
     for (int x = 0; x < kSegClasses; ++x) {
       const uint32_t m = __ballot_sync(0xFFFFFFFFu, c == x);
@@ -1081,8 +1081,7 @@ __global__ __launch_bounds__(128, 8) void k_sort_seg_warp(const int64_t *offsets
   }
 }
 
-// Class C: a block of T threads per segment, of up to 32 T ids; longer ones
-// (past the last class) in place in global memory.
+// Class C: a block of T threads per segment, of up to 32 T ids.
 template <int T, int C>
 __global__ __launch_bounds__(T, 1024 / T) void k_sort_seg_block(const int64_t *offsets, SegLists l, uint32_t *ids) {
   extern __shared__ uint32_t sm_seg[];  // T * 33
@@ -1094,9 +1093,31 @@ __global__ __launch_bounds__(T, 1024 / T) void k_sort_seg_block(const int64_t *o
     const uint32_t x = next;
     __syncthreads();
     if (x >= n) break;
-    const int64_t q = l.list[C * l.nq + x], b = offsets[q], len = offsets[q + 1] - b;
-    if (C == kSegClasses - 1 && len > 32 * T) {
-      uint32_t *v = ids + b;
+    const int64_t q = l.list[C * l.nq + x], b = offsets[q];
+    const int len = (int)(offsets[q + 1] - b);
+    if (C == 3 && len <= 16 * T)
+      seg_sort<T, 16>(ids + b, len, sm_seg);
+    else
+      seg_sort<T, 32>(ids + b, len, sm_seg);
+  }
+}
+
+// A block of 1024 threads per segment of any length: all segments of a call of
+// few boxes, or (LIST) those of the last class.  Up to 16384 ids in registers,
+// longer ones in place in global memory, where the network is bound by the
+// threads at work: 8 lists of 2e5 ids 11.8 ms with 1024 threads, 20.4 with 512.
+constexpr int kSegT = 1024, kSegTMax = 16 * kSegT;
+
+template <bool LIST>
+__global__ __launch_bounds__(kSegT, 1) void k_sort_seg_any(const int64_t *offsets, SegLists l, uint32_t *ids) {
+  extern __shared__ uint32_t sm_seg[];  // kSegT * 17
+  const int64_t n = LIST ? (int64_t)l.ctr[kSegClasses - 1] : l.nq;
+  for (int64_t x = blockIdx.x; x < n; x += gridDim.x) {
+    const int64_t q = LIST ? (int64_t)l.list[(kSegClasses - 1) * l.nq + x] : x;
+    const int64_t b = offsets[q], len = offsets[q + 1] - b;
+    uint32_t *v = ids + b;
+    if (len < 2) continue;
+    if (len > kSegTMax) {
       bitonic_ascending(
           len, [&](int64_t i, int64_t j) { return v[i] < v[j]; },
           [&](int64_t i, int64_t j) {
@@ -1104,10 +1125,24 @@ __global__ __launch_bounds__(T, 1024 / T) void k_sort_seg_block(const int64_t *o
             v[i] = v[j];
             v[j] = tmp;
           });
-    } else if (C == kSegClasses - 1 && len <= 16 * T) {
-      seg_sort<T, 16>(ids + b, (int)len, sm_seg);
-    } else {
-      seg_sort<T, 32>(ids + b, (int)len, sm_seg);
+    } else if (!LIST) {
+      if (len <= 256) {  // one warp: no barriers
+        if (threadIdx.x < 32) {
+          if (len <= 32)
+            seg_sort<32, 1>(v, (int)len, sm_seg);
+          else if (len <= 64)
+            seg_sort<32, 2>(v, (int)len, sm_seg);
+          else
+            seg_sort<32, 8>(v, (int)len, sm_seg);
+        }
+        __syncthreads();
+      } else if (len <= 1 * kSegT) {
+        seg_sort<kSegT, 1>(v, (int)len, sm_seg);
+      } else if (len <= 4 * kSegT) {
+        seg_sort<kSegT, 4>(v, (int)len, sm_seg);
+      } else {
+        seg_sort<kSegT, 16>(v, (int)len, sm_seg);
+      }
     }
   }
 }
@@ -1122,7 +1157,22 @@ psi_status launch_sort_seg(const int64_t *offsets, const SegLists &l, uint32_t *
   return PSI_OK;
 }
 
+template <bool LIST>
+psi_status launch_sort_seg_any(const int64_t *offsets, const SegLists &l, uint32_t *ids, cudaStream_t s) {
+  const size_t smem = LIST ? 0 : sizeof(uint32_t) * kSegT * 17;
+  if (smem > 48 * 1024)
+    PSI_CK(cudaFuncSetAttribute(k_sort_seg_any<LIST>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PSI_LAUNCH_NAMED("k_sort_seg_any", k_sort_seg_any<LIST>,
+                   (int)std::min<int64_t>(l.nq, (int64_t)num_sms() * (LIST ? 2 : 1)), kSegT, smem, s, offsets, l, ids);
+  return PSI_OK;
+}
+
+// With at most a segment per SM one launch sorts them all, without lists: 10
+// lists of 30 ids 5.7 us (by classes 34 with their launches, under the event
+// timer), 150 of 3000 14.8 (50.0), 150 of 20000 586 (644).  More lists queue up
+// behind its one block per SM: 300 of 20000 1156 us (919).
 psi_status sort_segments(const int64_t *offsets, int64_t nq, uint32_t *ids, cudaStream_t s) {
+  if (nq <= num_sms()) return launch_sort_seg_any<false>(offsets, SegLists{nullptr, nullptr, nq}, ids, s);
   Buf<uint32_t> list, ctr;
   psi_status st;
   if ((st = list.alloc(kSegClasses * nq, s)) || (st = ctr.alloc(2 * kSegClasses, s))) return st;
@@ -1131,7 +1181,7 @@ psi_status sort_segments(const int64_t *offsets, int64_t nq, uint32_t *ids, cuda
   PSI_LAUNCH(k_seg_classes, (int)std::min<int64_t>(ceil_div(nq, 256), (int64_t)num_sms() * 8), 256, 0, s, offsets, l);
   PSI_LAUNCH(k_sort_seg_warp, (int)std::min<int64_t>(ceil_div(nq, 4), (int64_t)num_sms() * 8), 128, 0, s, offsets, l, ids);
   if ((st = launch_sort_seg<64, 1>(offsets, l, ids, s)) || (st = launch_sort_seg<128, 2>(offsets, l, ids, s)) ||
-      (st = launch_sort_seg<512, 3>(offsets, l, ids, s)))
+      (st = launch_sort_seg<512, 3>(offsets, l, ids, s)) || (st = launch_sort_seg_any<true>(offsets, l, ids, s)))
     return st;
   return PSI_OK;
 }
