@@ -243,6 +243,7 @@ __global__ __launch_bounds__(LT, K <= 10 ? (D == 2 ? 8 : 7) : 6) void k_knn_lane
   // (P-Orth), the narrowest one's of the leaf and its neighbours (SPaC).
   float diag = 0.0f;
   uint32_t wlo = 1u, whi = 0u;  // P-Orth: the seeds' slots [wlo, whi)
+  bool hard = false;
   if (hi >= lo) diag = box_diag2<D>(t, PORTH ? (uint32_t)sd.leaf_node[j] : (uint32_t)j);
   S.init(a.k, diag);
   {
@@ -277,20 +278,21 @@ __global__ __launch_bounds__(LT, K <= 10 ? (D == 2 ? 8 : 7) : 6) void k_knn_lane
         up = hi + 1 < le && (up || !right);
         down = lo > lb && (down || right);
       }
-      if (PORTH)
-        S.bound_by(wlo, (int)(whi - wlo));
-      else
+      if (PORTH) {
+        hard = whi - wlo > kCntMask;  // a pile of duplicate points: one lane alone would walk it all
+        if (!hard) S.bound_by(wlo, (int)(whi - wlo));
+      } else {
         for (int x = lo; x <= hi; ++x) S.bound_by(t.ref[x], t.cnt[x]);
+      }
     }
     __syncwarp();
     S.set_bound();
   }
   uint32_t kdk = order_key(S.kb);
-  int seen = lo;              // next of the leaves [alo, ahi] that are in F but not noted
   const int seen_end = hi;
+  int seen = hard ? hi + 1 : lo;  // next of the seed leaves, which are in F but not noted
   int np = 0;     // pairs waiting (warp-uniform)
   int total = 0;  // leaves this query has put in the pool in its search
-  bool hard = false;
 
   // The leaves just before and after the seeds, where they may hold a
   // neighbour (SPaC): a seed leaf that spans a jump of the curve (or a gap
@@ -347,10 +349,8 @@ __global__ __launch_bounds__(LT, K <= 10 ? (D == 2 ? 8 : 7) : 6) void k_knn_lane
         c = PORTH ? (int)(whi - wlo) : t.cnt[seen];
         seen = PORTH ? seen_end + 1 : seen + 1;
       }
-      const bool pile = PORTH && c > (int)kCntMask;  // of duplicate points
-      hard |= pile;
-      const uint32_t nm = __ballot_sync(0xFFFFFFFFu, need && !pile);
-      if (need && !pile) s_pool[w][__popc(nm & lanemask_lt())] = make_uint2(s0, pair_word(0, lane, c));
+      const uint32_t nm = __ballot_sync(0xFFFFFFFFu, need);
+      if (need) s_pool[w][__popc(nm & lanemask_lt())] = make_uint2(s0, pair_word(0, lane, c));
       np = __popc(nm);
     } else if (stage == 2) {
       for (;;) {
