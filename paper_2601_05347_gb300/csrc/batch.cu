@@ -1021,7 +1021,7 @@ static psi_status batch_knn(psi_batch *b, const int32_t *d_q, const int64_t *d_q
   hard.q = seed.pos + nq;  // the other half of that buffer, and the sort's free position buffer
   hard.pos = r.vals == b->qv0 ? b->qv1 : b->qv0;
   hard.n = b->d_nhard;
-  return run_knn_roots(tv, d_q, nq, k, r.vals, b->d_qroot, b->D, d_ids, d_d2, b->d_status, d_stats, s, seed, -1, false,
+  return run_knn_roots(tv, b->total, d_q, nq, k, r.vals, b->d_qroot, b->D, d_ids, d_d2, b->d_status, d_stats, s, seed, -1, false,
                        hard);
 }
 

@@ -18,6 +18,7 @@
 // Range list: the same traversal counts first; after an exclusive scan of the
 // counts a second traversal writes each query's ids at its offset (a
 // subtree inside the box is enumerated without further box tests).
+#include <cmath>
 #include <type_traits>
 
 #include "bitonic.cuh"
@@ -1227,30 +1228,48 @@ psi_status query_order(const psi_index *ix, const int32_t *q, int64_t nq, QueryO
   return PSI_OK;
 }
 
-// Fewest queries for which the one-query-per-thread kernel is the faster one:
-// it needs the chip full of queries (a wave is 8 blocks of 128 per SM), more
-// of them the longer the lists and, on P-Orth, the more nodes its shared walk
-// visits.  Measured on 1e7 points, whole call, warp per query / this kernel, in
-// us: 2D SPaC-H 10-NN 1.5e5 queries 390 / 351, 3e5 642 / 458, 1e6 1707 / 923;
-// 3D uniform SPaC-H 10-NN 1.5e5 546 / 523, 1e6 2520 / 1477; 3D P-Orth 10-NN
-// 3e5 1752 / 1686, 1e6 4553 / 3271, 16-NN 3e5 2278 / 2796.
-static int64_t lane_min_queries(int D, int k, bool porth) {
-  const int64_t wave = (int64_t)num_sms() * 1024;
-  if (k > kLaneMaxK || (porth && D == 3 && k > 10)) return INT64_MAX;
-  if (!porth) return k <= 5 ? wave : k <= 10 ? wave * 3 / 2 : D == 2 ? wave * 2 : wave * 3;
-  if (k == 1) return wave;
-  if (D == 2) return k <= 10 ? wave * 2 : wave * 4;
-  return k <= 5 ? wave * 5 / 2 : wave * 4;
+// Fewest queries for which the one-query-per-thread kernel is the faster one,
+// over n points on a chip of sms multiprocessors.  It needs the chip full of
+// queries (a wave is 8 blocks of 128 per SM), more of them the longer the lists
+// and, above some 3e6 points, the farther apart the queries of a warp are, whose
+// shared walk is the longer.  The lines are read from 8e3 timings, 3e5 to 1e8
+// points, uniform and Varden, 2e4 to 2e6 queries.  Other kernel / this one, in
+// us, 10-NN at data points: 2D SPaC-H 3e5 queries on 3e6 points 562 / 395, on 1e8
+// 706 / 732, 1e6 on 1e8 2072 / 1340; 3D SPaC-H 3e5 on 3e5 710 / 464, on 1e8 1141 /
+// 1486, 1e6 on 1e8 3348 / 3025; 3D P-Orth 6e5 on 3e6 2014 / 1196, on 3e7 2364 /
+// 2218.  A batch's other kernel takes one query per warp and is ahead for longer
+// in 3D: 64 indexes of 1e6 uniform points, 10-NN of 4.7e5 queries 1484 / 1604, of
+// 1.2e6 3906 / 2913 (Varden 1616 / 2474, 4187 / 5319).
+static int64_t lane_min_queries(int sms, int D, int k, bool porth, bool batch, int64_t n) {
+  if (k > kLaneMaxK) return INT64_MAX;
+  // [P-Orth][D - 2]: waves at 3e6 points by k, and the exponent of the points
+  static constexpr struct {
+    double k1, k5, k10, k13, k16, c;
+  } kFit[2][2] = {{{0.33, 0.36, 0.55, 0.8, 0.8, 0.35}, {0.38, 0.5, 0.85, 1.5, 1.5, 0.38}},
+                  {{0.3, 0.35, 0.45, 0.9, 1.2, 0.3}, {0.33, 0.6, 1.1, 1.6, 3.0, 0.33}}};
+  const auto &f = kFit[porth][D - 2];
+  double waves = k == 1 ? f.k1 : k <= 5 ? f.k5 : k <= 10 ? f.k10 : k <= 13 ? f.k13 : f.k16;
+  waves *= std::pow(std::max(1.0, (double)n / 3e6), f.c);
+  if (batch && D == 3) waves *= 1.2;
+  // (P-Orth queries away from the data are only listed here: at one wave the
+  // whole call is 0.80 to 0.89 times as fast, at two 0.85 to 1)
+  return (int64_t)((double)sms * 1024 * std::max(waves, porth && k > 1 ? 1.9 : 1.0));
 }
 
-// On P-Orth, one query per warp with small leaves scanned together beats two
-// queries per warp with one leaf at a time, except where the lists are short
-// and there are many queries.  10-NN, two per warp / one, in us: 3D uniform 5e3
-// queries 257 / 108, 1e5 759 / 632 (32-NN 1473 / 937); 2D Varden 5e3 203 / 99,
-// 1e5 533 / 592 (32-NN 857 / 753).
-static bool porth_single(int D, int k, int64_t nq) { return k > (D == 3 ? 8 : 16) || (nq < 32768 && k > 4); }
+// On P-Orth, one query per warp with small leaves scanned together, for few
+// queries (the chip is not full, a query's latency counts), long lists and large
+// trees; else two queries per warp with one leaf at a time.  The line is fitted
+// to the same timings.  Two per warp / one, in us, at data points: 3D uniform 3e6
+// points 10-NN 2e4 queries 165 / 130, 6e5 2014 / 2403; 3D Varden 3e5 points 10-NN
+// 6e5 2082 / 3034; 3D uniform 1e8 points 32-NN 2e4 1023 / 256, 6e5 8781 / 5345.
+static int64_t porth_single_max(int D, int k, int64_t n) {
+  const double m = (double)n / 1e6;
+  const double line = D == 2 ? 7450 * std::pow((double)k, 0.7) * std::pow(m, 0.3) : 5960 * k * std::pow(std::max(m, 0.6), 0.6);
+  return (int64_t)std::max(line, 12000.0);
+}
+static bool porth_single(int D, int k, int64_t nq, int64_t n) { return nq < porth_single_max(D, k, n); }
 
-psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k, const uint32_t *order,
+psi_status run_knn_roots(const TreeView &tv, int64_t n, const int32_t *q, int64_t nq, int k, const uint32_t *order,
                          const int32_t *qroot, int D, uint32_t *out_id, int64_t *out_d2, int *status,
                          unsigned long long *d_stats, cudaStream_t s, const KnnSeed &seed, int64_t leaf_limit,
                          bool porth, const KnnHard &hard) {
@@ -1265,7 +1284,7 @@ psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k
     const int gs = (int)std::max<int64_t>(1, std::min<int64_t>(ceil_div(nq, 256), (int64_t)num_sms() * 16));
     PSI_LAUNCH(k_knn_seed, gs, 256, 0, s, seed, tv.ref, order, nq, seed.pos);
   }
-  if (hard.q && !d_stats && nq >= lane_min_queries(D, k, porth)) {
+  if (hard.q && !d_stats && nq >= lane_min_queries(num_sms(), D, k, porth, qroot != nullptr, n)) {
     PSI_CK(cudaMemsetAsync(hard.n, 0, sizeof(uint32_t), s));
     LaneArgs l{a, hard.q, hard.pos, hard.n};
     psi_status st = run_knn_lane(l, D, porth, s);
@@ -1276,7 +1295,7 @@ psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k
     a.d_nq = hard.n;
 #define KNN_LIST(DD, PP)                                                                                            \
   do {                                                                                                              \
-    if (qroot || (porth && porth_single(D, k, nq)))                                                                  \
+    if (qroot || (porth && k > (D == 3 ? 8 : 16)))                                                                 \
       PSI_LAUNCH_NAMED("k_knn", (k_knn<DD, 1, false, PP, true>),                                                    \
                        resident_query_grid(k_knn<DD, 1, false, PP, true>, nq), QW * 32, 0, s, a, stats);            \
     else                                                                                                            \
@@ -1297,7 +1316,7 @@ psi_status run_knn_roots(const TreeView &tv, const int32_t *q, int64_t nq, int k
   }
   const int kpl = k <= 32 ? 1 : (k <= 64 ? 2 : 4);
   // k <= 32 over one tree with queries in curve order: kGroup queries per warp
-  if (kpl == 1 && !qroot && order && kGroup > 1 && !(porth && porth_single(D, k, nq))) {
+  if (kpl == 1 && !qroot && order && kGroup > 1 && !(porth && porth_single(D, k, nq, n))) {
 #define KNN_GROUP(DD, RC)                                                                                   \
   do {                                                                                                      \
     if (d_stats)                                                                                            \
@@ -1423,7 +1442,7 @@ psi_status run_knn(const psi_index *ix, const int32_t *q, int64_t nq, int k, uin
     seed.sep_key = ix->sep_key;
     seed.L = ix->L;
   }
-  return run_knn_roots(ix->view(), q, nq, k, qo.order, nullptr, ix->D, out_id, out_d2, ix->d_status, d_stats, s,
+  return run_knn_roots(ix->view(), ix->n, q, nq, k, qo.order, nullptr, ix->D, out_id, out_d2, ix->d_status, d_stats, s,
                        seed, ix->cfg.kind == PSI_PORTH ? -1 : ix->L, ix->cfg.kind == PSI_PORTH, hard);
 }
 
@@ -1457,3 +1476,12 @@ psi_status run_range_emit(const psi_index *ix, const int32_t *boxes, int64_t nq,
 }
 
 }  // namespace psi
+
+// Test hook of the rules above: the kernel that psi_knn chooses for queries in
+// curve order on one index ('L' one query per thread, 'S' one per warp, 'G' two).
+extern "C" int32_t psi_test_knn_form(int32_t dim, int32_t k, int32_t porth, int64_t nq, int64_t n, int32_t sms) {
+  using namespace psi;
+  if (nq >= lane_min_queries(sms, dim, k, porth != 0, false, n)) return 'L';
+  if (k > 32 || (porth && porth_single(dim, k, nq, n))) return 'S';
+  return 'G';
+}

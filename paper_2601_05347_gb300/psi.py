@@ -71,6 +71,7 @@ def lib():
             "psi_knn_instrumented": (st, [P, P, i64, i32, P, P, P, P]),
             "psi_sort_pairs_noalloc": (st, [P, P, i64, i32, P]),
             "psi_test_sort_withheld_tile": (st, [P, P, i64, i64, ctypes.c_uint32, P]),
+            "psi_test_knn_form": (i32, [i32, i32, i32, i64, i64, i32]),
             "psi_batch_create": (st, [P, P, i32, i32, P, P]),
             "psi_batch_device_wide": (i32, [P, P, i32, i32]),
             "psi_batch_build": (st, [P, P, P, P]),
