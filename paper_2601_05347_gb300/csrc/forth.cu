@@ -625,7 +625,8 @@ struct FKnnArgs {
   uint32_t *out_id;
   double *out_d2;
   int *status;
-  const uint32_t *d_nq = nullptr;  // listed queries (order): their number, at most nq
+  // listed queries (order): their number, at most nq, and the order of all nq
+  const uint32_t *d_nq = nullptr, *all_order = nullptr;
 };
 
 // One warp per query: depth-first search entering the nearest unvisited child
@@ -637,9 +638,17 @@ __global__ __launch_bounds__(FQW * 32) void k_fknn(FKnnArgs a) {
   __shared__ uint32_t s_c0[FQW][FMAXLVL], s_mask[FQW][FMAXLVL], s_leaf[FQW][FMAXLVL];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const FView &t = a.t;
-  const int64_t nq = LIST ? (int64_t)*a.d_nq : a.nq;
+  const uint32_t *order = a.order;
+  int64_t nq = a.nq;
+  if (LIST) {
+    nq = (int64_t)*a.d_nq;
+    if (4 * nq >= 3 * a.nq) {  // most of them: all, in curve order (as KnnTake)
+      order = a.all_order;
+      nq = a.nq;
+    }
+  }
   for (int64_t qi = (int64_t)blockIdx.x * FQW + w; qi < nq; qi += (int64_t)gridDim.x * FQW) {
-    const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
+    const int64_t q = order ? (int64_t)order[qi] : qi;
     float qc[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) qc[d] = a.q[q * D + d];
@@ -1254,6 +1263,7 @@ psi_status forth_knn_d(const psi_forth *ix, const float *q, int64_t nq, int k, u
       PSI_LAUNCH_NAMED("k_fknn", (k_fknn_lane<D, 10>), gl, FLT, 0, s, l);
     else
       PSI_LAUNCH_NAMED("k_fknn", (k_fknn_lane<D, 16>), gl, FLT, 0, s, l);
+    a.all_order = order;
     a.order = l.hq;
     a.d_nq = l.hn;
     PSI_LAUNCH_NAMED("k_fknn", (k_fknn<D, 1, true>), g, FQW * 32, 0, s, a);

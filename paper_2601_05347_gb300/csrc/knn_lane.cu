@@ -244,7 +244,13 @@ __global__ __launch_bounds__(LT, K <= 10 ? (D == 2 ? 8 : 7) : 6) void k_knn_lane
   float diag = 0.0f;
   uint32_t wlo = 1u, whi = 0u;  // P-Orth: the seeds' slots [wlo, whi)
   bool hard = false;
-  if (hi >= lo) diag = box_diag2<D>(t, PORTH ? (uint32_t)sd.leaf_node[j] : (uint32_t)j);
+  // lower bounds of the squared distances to the seeds and (SPaC) to the leaves beside them
+  uint32_t skey = 0x7F800000u, nkey[2] = {0x7F800000u, 0x7F800000u};
+  if (hi >= lo) {
+    const uint32_t nd = PORTH ? (uint32_t)sd.leaf_node[j] : (uint32_t)j;
+    diag = box_diag2<D>(t, nd);
+    skey = lane_box_key<D>(t, nd, S.qc);
+  }
   S.init(a.k, diag);
   {
     const int want = PORTH ? (K == 1 ? 4 : max(a.k, kSeedPoints)) : a.k;
@@ -273,16 +279,28 @@ __global__ __launch_bounds__(LT, K <= 10 ? (D == 2 ? 8 : 7) : 6) void k_knn_lane
             wlo = r;
           diag = fmaxf(diag, box_diag2<D>(t, e));
         }
+        skey = min(skey, lane_box_key<D>(t, e, S.qc));
         (right ? hi : lo) = nx;
         got += c;
         up = hi + 1 < le && (up || !right);
         down = lo > lb && (down || right);
       }
       if (PORTH) {
-        hard = whi - wlo > kCntMask;  // a pile of duplicate points: one lane alone would walk it all
+        // a pile of duplicate points, which one lane alone would walk, or seeds
+        // whose boxes already show that they are far from the query
+        hard = whi - wlo > kCntMask || __uint_as_float(skey) > kLoose * diag;
         if (!hard) S.bound_by(wlo, (int)(whi - wlo));
       } else {
-        for (int x = lo; x <= hi; ++x) S.bound_by(t.ref[x], t.cnt[x]);
+        for (int side = 0; side < 2; ++side) {
+          const int nb = side ? hi + 1 : lo - 1;
+          if (nb < lb || nb >= le) continue;
+          diag = fminf(diag, box_diag2<D>(t, (uint32_t)nb));
+          nkey[side] = lane_box_key<D>(t, (uint32_t)nb, S.qc);
+        }
+        const float far = kLoose * diag;
+        hard = __uint_as_float(min(skey, min(nkey[0], nkey[1]))) > far;
+        if (!hard)
+          for (int x = lo; x <= hi; ++x) S.bound_by(t.ref[x], t.cnt[x]);
       }
     }
     __syncwarp();
@@ -290,7 +308,6 @@ __global__ __launch_bounds__(LT, K <= 10 ? (D == 2 ? 8 : 7) : 6) void k_knn_lane
   }
   uint32_t kdk = order_key(S.kb);
   const int seen_end = hi;
-  int seen = hard ? hi + 1 : lo;  // next of the seed leaves, which are in F but not noted
   int np = 0;     // pairs waiting (warp-uniform)
   int total = 0;  // leaves this query has put in the pool in its search
 
@@ -298,31 +315,24 @@ __global__ __launch_bounds__(LT, K <= 10 ? (D == 2 ? 8 : 7) : 6) void k_knn_lane
   // neighbour (SPaC): a seed leaf that spans a jump of the curve (or a gap
   // between clusters) gives the queries beside it a bound as wide as the jump,
   // and the leaf on their side of it the true one.
+  int seen = lo;  // next of the seed leaves, which are in F but not noted
   if (!PORTH) {
-    uint32_t skey[2] = {0x7F800000u, 0x7F800000u};
-    for (int side = 0; side < 2; ++side) {
-      const int nb = side ? hi + 1 : lo - 1;
-      if (hi >= lo && nb >= lb && nb < le) {
-        diag = fminf(diag, box_diag2<D>(t, (uint32_t)nb));
-        skey[side] = lane_box_key<D>(t, (uint32_t)nb, S.qc);
-      }
-    }
     // a query away from the data: neither the seeds nor the leaves beside them
     // are near it on their own scale
     const float far = kLoose * diag;
-    hard = hi >= lo && __uint_as_float(kdk) > far && __uint_as_float(skey[0]) > far && __uint_as_float(skey[1]) > far;
-    if (hard) seen = seen_end + 1;
+    hard |= hi >= lo && __uint_as_float(kdk) > far && __uint_as_float(min(nkey[0], nkey[1])) > far;
     for (int side = 0; side < 2; ++side) {
-      const bool need = !hard && hi >= lo && skey[side] < 0x7F800000u && skey[side] <= kdk;
+      const bool need = !hard && hi >= lo && nkey[side] < 0x7F800000u && nkey[side] <= kdk;
       const uint32_t nm = __ballot_sync(0xFFFFFFFFu, need);
       if (need) {
         const int nb = side ? hi + 1 : lo - 1;
-        s_pool[w][np + __popc(nm & lanemask_lt())] = make_uint2(t.ref[nb], pair_word(skey[side], lane, t.cnt[nb]));
+        s_pool[w][np + __popc(nm & lanemask_lt())] = make_uint2(t.ref[nb], pair_word(nkey[side], lane, t.cnt[nb]));
         (side ? hi : lo) = nb;
       }
       np += __popc(nm);
     }
   }
+  if (hard) seen = seen_end + 1;
   // SPaC: the seeds as node numbers [slo, shi]
   const uint32_t slo = hi >= lo ? (uint32_t)lo : 1u, shi = hi >= lo ? (uint32_t)hi : 0u;
 

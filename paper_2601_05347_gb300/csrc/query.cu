@@ -197,7 +197,8 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   KWait *wt = &s_wait[KPL > 1 ? w : 0];
   const int64_t warps = (int64_t)gridDim.x * QW;
-  const int64_t nq = LIST ? (int64_t)*a.d_nq : a.nq;
+  const KnnTake take(a, LIST);
+  const int64_t nq = take.nq;
   const TreeView &t = a.t;
   __shared__ alignas(16) uint8_t s_tab[SELF ? kCurveTabBytes : 16];
   if (SELF && a.seed.curve == CURVE_HILBERT) {
@@ -206,7 +207,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
   }
   unsigned long long n_int = 0, n_leaf = 0, n_pts = 0, n_kids = 0;
   for (int64_t qi = (int64_t)blockIdx.x * QW + w; qi < nq; qi += warps) {
-    const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
+    const int64_t q = take.order ? (int64_t)take.order[qi] : qi;
     int32_t qc[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) qc[d] = a.q[q * D + d];
@@ -231,7 +232,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
       s_lo = s_hi = seed_search_warp(sd.sep_key, sd.L, key);
       knn_scan_leaf<D, KPL, true>(t, (uint32_t)s_lo, qc, kl, wt, nw, a.k);
     } else if (sd.qkey && root >= 0) {
-      const int64_t pos = sd.pos[qi];  // k_knn_seed
+      const int64_t pos = take.pos[qi];  // k_knn_seed
       if (L > 0) {
         // P-Orth: pos is a position in the key-ordered leaf list
         const int64_t j = sd.leaf_node ? (int64_t)sd.leaf_node[pos] : pos;
@@ -444,9 +445,9 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
           // WIDE: the top entries, one per group of lanes, while the stack has
           // room for the most that single pops may add (2^D - 1 per level)
           while (WIDE && sp > 0 && !more) {
-            const int g = lane / CW, take = sp <= 64 ? min(sp, 32 / CW) : 1;
-            e = g < take ? s_stk[w][sp - 1 - g] : make_uint4(0, 0xFFFFFFFFu, 0, 0);
-            sp -= take;
+            const int g = lane / CW, pops = sp <= 64 ? min(sp, 32 / CW) : 1;
+            e = g < pops ? s_stk[w][sp - 1 - g] : make_uint4(0, 0xFFFFFFFFu, 0, 0);
+            sp -= pops;
             if (e.y > kdk) e = make_uint4(0, 0, 0, 0);  // no children
             more = __any_sync(0xFFFFFFFFu, e.w != 0);
           }
@@ -542,7 +543,8 @@ __global__ __launch_bounds__(QW * 32) void k_knn_group(KnnArgs a, KnnStats stats
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const TreeView &t = a.t;
   const KnnSeed &sd = a.seed;
-  const int64_t nq = LIST ? (int64_t)*a.d_nq : a.nq;
+  const KnnTake take(a, LIST);
+  const int64_t nq = take.nq;
   const int64_t ngroups = (nq + G - 1) / G;
   unsigned long long n_int = 0, n_leaf = 0, n_pts = 0, n_kids = 0;
   for (int64_t gi = (int64_t)blockIdx.x * QW + w; gi < ngroups; gi += (int64_t)gridDim.x * QW) {
@@ -553,10 +555,10 @@ __global__ __launch_bounds__(QW * 32) void k_knn_group(KnnArgs a, KnnStats stats
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       const int64_t qi = qi0 + min(g, ng - 1);  // a short last group repeats its last query
-      const int64_t q = a.order ? (int64_t)a.order[qi] : qi;
+      const int64_t q = take.order ? (int64_t)take.order[qi] : qi;
 #pragma unroll
       for (int d = 0; d < D; ++d) qc[g][d] = a.q[q * D + d];
-      seed[g] = !sd.qkey ? 0xFFFFFFFFu : sd.leaf_node ? (uint32_t)sd.leaf_node[sd.pos[qi]] : sd.pos[qi];
+      seed[g] = !sd.qkey ? 0xFFFFFFFFu : sd.leaf_node ? (uint32_t)sd.leaf_node[take.pos[qi]] : take.pos[qi];
     }
     KList<1> kl[G];
 #pragma unroll
@@ -744,7 +746,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn_group(KnnArgs a, KnnStats stats
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       if (g < ng && lane < a.k) {
-        const int64_t q = a.order ? (int64_t)a.order[qi0 + g] : qi0 + g;
+        const int64_t q = take.order ? (int64_t)take.order[qi0 + g] : qi0 + g;
         a.out_id[q * a.k + lane] = kl[g].i[0];
         a.out_d2[q * a.k + lane] = kl[g].d[0];
       }
@@ -1289,19 +1291,31 @@ psi_status run_knn_roots(const TreeView &tv, int64_t n, const int32_t *q, int64_
     LaneArgs l{a, hard.q, hard.pos, hard.n};
     psi_status st = run_knn_lane(l, D, porth, s);
     if (st) return st;
-    // the queries it left out, a warp for each (or for two)
+    // the queries it left out, a warp for each or (SPaC, and long lists on P-Orth,
+    // where neighbours on the list are rarely neighbours in space) for two: their
+    // number is known on the device only, so on P-Orth both kernels are launched
+    // and one of them finds nothing to do
+    a.all_order = order;
+    a.all_pos = seed.pos;
     a.order = hard.q;
     a.seed.pos = hard.pos;
     a.d_nq = hard.n;
 #define KNN_LIST(DD, PP)                                                                                            \
   do {                                                                                                              \
-    if (qroot || (porth && k > (D == 3 ? 8 : 16)))                                                                 \
-      PSI_LAUNCH_NAMED("k_knn", (k_knn<DD, 1, false, PP, true>),                                                    \
-                       resident_query_grid(k_knn<DD, 1, false, PP, true>, nq), QW * 32, 0, s, a, stats);            \
-    else                                                                                                            \
-      PSI_LAUNCH_NAMED("k_knn", (k_knn_group<DD, kGroup, false, PP, true>),                                         \
+    const int64_t split = PP ? 3 * porth_single_max(D, k, n) : qroot ? INT64_MAX : 0;                                \
+    if (split > 0) {                                                                                                 \
+      a.list_lo = 0;                                                                                                 \
+      a.list_hi = split;                                                                                             \
+      PSI_LAUNCH_NAMED("k_knn", (k_knn<DD, 1, false, PP, true>),                                                     \
+                       resident_query_grid(k_knn<DD, 1, false, PP, true>, nq), QW * 32, 0, s, a, stats);             \
+    }                                                                                                                \
+    if (split < INT64_MAX) {                                                                                         \
+      a.list_lo = split;                                                                                             \
+      a.list_hi = INT64_MAX;                                                                                         \
+      PSI_LAUNCH_NAMED("k_knn", (k_knn_group<DD, kGroup, false, PP, true>),                                          \
                        resident_query_grid(k_knn_group<DD, kGroup, false, PP, true>, ceil_div(nq, kGroup)), QW * 32, \
-                       0, s, a, stats);                                                                             \
+                       0, s, a, stats);                                                                              \
+    }                                                                                                                \
   } while (0)
     if (D == 2) {
       if (porth) KNN_LIST(2, true);
