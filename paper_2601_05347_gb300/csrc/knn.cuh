@@ -36,6 +36,9 @@ __device__ __forceinline__ uint32_t order_key(int64_t md) {
   return __float_as_uint(__fmaf_ru(__uint2float_ru(hi), 4294967296.0f, __uint2float_ru(lo)));
 }
 
+// order_key of the k-th distance of a list that is not full yet.
+constexpr uint32_t kNoBound = 0x5F000000u;
+
 struct KnnArgs {
   TreeView t;
   const int32_t *q;

@@ -442,10 +442,11 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
           expand(c0, nk, pl, pkey);
           uint4 e = make_uint4(0, 0, 0, 0);
           bool more = false;
-          // WIDE: the top entries, one per group of lanes, while the stack has
-          // room for the most that single pops may add (2^D - 1 per level)
+          // WIDE: the top entries, one per group of lanes, once the list is full
+          // and while the stack has room for the most that single pops may add
+          // (2^D - 1 per level)
           while (WIDE && sp > 0 && !more) {
-            const int g = lane / CW, pops = sp <= 64 ? min(sp, 32 / CW) : 1;
+            const int g = lane / CW, pops = sp <= 64 && kdk < kNoBound ? min(sp, 32 / CW) : 1;
             e = g < pops ? s_stk[w][sp - 1 - g] : make_uint4(0, 0xFFFFFFFFu, 0, 0);
             sp -= pops;
             if (e.y > kdk) e = make_uint4(0, 0, 0, 0);  // no children
@@ -1377,10 +1378,12 @@ psi_status run_knn_roots(const TreeView &tv, int64_t n, const int32_t *q, int64_
     return PSI_OK;
   }
   // Few queries on P-Orth leave the chip waiting on the chain of dependent node
-  // loads of each search: up to four nodes are expanded at once, at the price of
-  // some that single steps would have pruned (1e3 10-NN on 1e6 3D uniform
-  // points 29.3 -> 25.5 us a call; queries away from 1e7 3D Varden points 123
-  // -> 104 us).
+  // loads of each search: once a query's list is full, up to four nodes are
+  // expanded at once, at the price of some that single steps would have pruned.
+  // Before that there is no bound and the nearest node is the one wanted: four at
+  // once from the start took 18.5 us for 4e3 1-NN at data points of 1e6 3D uniform
+  // points, single steps 14.4.  Over 2D and 3D, 3e4 to 2e7 points, 1 to 4e3 queries
+  // at, near and away from the data: 1.00 to 1.38 times as fast as single steps.
   if (porth && kpl == 1 && !order && !d_stats) {
     if (D == 2)
       PSI_LAUNCH_NAMED("k_knn", (k_knn<2, 1, false, true, false, false, true>),
