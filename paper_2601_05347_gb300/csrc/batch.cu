@@ -51,6 +51,7 @@ struct psi_batch {
   int64_t *d_qoff = nullptr;
   uint64_t *qk0 = nullptr, *qk1 = nullptr;
   uint32_t *qv0 = nullptr, *qv1 = nullptr;
+  uint32_t *q_scratch = nullptr;  // of the sort of the queries
   uint32_t *d_nhard = nullptr;  // queries the k-NN's first kernel leaves to the second
   cudaStream_t last_stream = nullptr;
 };
@@ -727,7 +728,7 @@ static void batch_free(psi_batch *b) {
                   (void *)b->d_root, (void *)b->d_queue, (void *)b->d_status, (void *)b->kA, (void *)b->kB,
                   (void *)b->vA, (void *)b->vB, (void *)b->d_qroot, (void *)b->d_qseg, (void *)b->d_qoff,
                   (void *)b->qk0, (void *)b->qk1, (void *)b->qv0, (void *)b->qv1, (void *)b->d_nhard,
-                  (void *)b->sort_scratch})
+                  (void *)b->sort_scratch, (void *)b->q_scratch})
     DevMem::free(p, s);
   delete b;
 }
@@ -940,12 +941,12 @@ psi_status psi_batch_knn_reserve(psi_batch *b, int64_t max_queries, void *stream
   if (max_queries <= b->q_cap) return PSI_OK;
   cudaStream_t s = (cudaStream_t)stream;
   for (void *p : {(void *)b->d_qroot, (void *)b->d_qseg, (void *)b->d_qoff, (void *)b->qk0, (void *)b->qk1,
-                  (void *)b->qv0, (void *)b->qv1})
+                  (void *)b->qv0, (void *)b->qv1, (void *)b->q_scratch})
     DevMem::free(p, s);
   b->d_qroot = b->d_qseg = nullptr;
   b->d_qoff = nullptr;
   b->qk0 = b->qk1 = nullptr;
-  b->qv0 = b->qv1 = nullptr;
+  b->qv0 = b->qv1 = b->q_scratch = nullptr;
   const size_t Q = (size_t)std::max<int64_t>(max_queries, 1);
   psi_status st;
   if ((st = DevMem::alloc((void **)&b->d_qroot, sizeof(int32_t) * Q, s)) ||
@@ -954,7 +955,8 @@ psi_status psi_batch_knn_reserve(psi_batch *b, int64_t max_queries, void *stream
       (st = DevMem::alloc((void **)&b->qk0, sizeof(uint64_t) * Q, s)) ||
       (st = DevMem::alloc((void **)&b->qk1, sizeof(uint64_t) * Q, s)) ||
       (st = DevMem::alloc((void **)&b->qv0, sizeof(uint32_t) * Q, s)) ||
-      (st = DevMem::alloc((void **)&b->qv1, sizeof(uint32_t) * Q, s)))
+      (st = DevMem::alloc((void **)&b->qv1, sizeof(uint32_t) * Q, s)) ||
+      (st = DevMem::alloc((void **)&b->q_scratch, sizeof(uint32_t) * sort_scratch_words((int64_t)Q), s)))
     return st;
   b->q_cap = max_queries;
   return PSI_OK;
@@ -994,7 +996,7 @@ static psi_status batch_knn(psi_batch *b, const int32_t *d_q, const int64_t *d_q
   SortResult r;
   EncodeSpec none;
   psi_status st = sort_pairs(none, b->qk0, b->qv0, nq, 40 + segbits, nullptr, b->qk1, b->qv1, b->qk0, b->qv0,
-                             b->d_status, s, &r);
+                             b->d_status, s, &r, 0, b->q_scratch);
   if (st) return st;
   TreeView tv;
   for (int d = 0; d < 3; ++d) {

@@ -59,3 +59,19 @@ def test_build_takes_no_memory(sizes, threads):
     assert (psi.launch_count() - n0 > 1) == (threads == 0)  # the form that was meant
     assert m.rise == 0
     b.sync()
+
+
+@pytest.mark.parametrize("reserved,asked", [(80001, 80000), (80001, 500), (200_000, 200_000), (200_000, 33)])
+def test_knn_takes_no_memory(reserved, asked):
+    b, pts, ids = batch([30000, 9], 0)
+    b.build(pts, ids)
+    b.reserve(reserved)
+    q = pts[torch.arange(asked, device="cuda") % len(pts)].contiguous()
+    qoff = torch.tensor([0, asked, asked], device="cuda")
+    for k in (10, 40):
+        out = torch.empty((asked, k), dtype=torch.int32, device="cuda"), torch.empty((asked, k), dtype=torch.int64,
+                                                                                      device="cuda")
+        with PoolHigh() as m:
+            b.knn(q, qoff, k, *out)
+        assert m.rise == 0
+    b.sync()
