@@ -943,6 +943,7 @@ psi_status psi_batch_knn_reserve(psi_batch *b, int64_t max_queries, void *stream
   for (void *p : {(void *)b->d_qroot, (void *)b->d_qseg, (void *)b->d_qoff, (void *)b->qk0, (void *)b->qk1,
                   (void *)b->qv0, (void *)b->qv1, (void *)b->q_scratch})
     DevMem::free(p, s);
+  b->q_cap = 0;  // nothing is reserved until all of it is
   b->d_qroot = b->d_qseg = nullptr;
   b->d_qoff = nullptr;
   b->qk0 = b->qk1 = nullptr;
