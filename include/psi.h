@@ -154,12 +154,14 @@ typedef struct psi_batch psi_batch;
  * point array: index i owns points [h_offsets[i], h_offsets[i+1]) (host array
  * of nidx+1 entries, h_offsets[0] = 0).  All indexes share cfg (SPAC_Z or
  * SPAC_H).  `threads` is the thread-block size of the build (256, 512, 1024; 0
- * = 512); cfg->radix_bits is the digit width of the build's block sort (0 or 8:
+ * leaves it open: 512); cfg->radix_bits is the digit width of the build's block sort (0 or 8:
  * 8-bit digits; 11: 11-bit digits, with 256 or 512 threads only).  The index
  * layout does not depend on either; with both 0, a batch whose points are mostly
  * in a few large indexes is built by device-wide sorts instead of a block per
- * index.  Allocates everything the build needs, so psi_batch_build and
- * psi_batch_knn allocate nothing and can be captured in a CUDA graph.
+ * index.  Allocates everything the build needs (with device-wide sorts, their
+ * look-back tables too: half a byte per point), and psi_batch_knn_reserve what
+ * the queries need, so psi_batch_build and psi_batch_knn allocate nothing and
+ * can be captured in a CUDA graph.
  * Synchronises `stream`. */
 psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int32_t nidx, int32_t threads,
                             void *stream, psi_batch **out);
@@ -168,10 +170,10 @@ psi_status psi_batch_create(const psi_config *cfg, const int64_t *h_offsets, int
 int32_t psi_batch_device_wide(const psi_config *cfg, const int64_t *h_offsets, int32_t nidx, int32_t threads);
 
 /* Builds every index of the batch (Algorithm 3 per index: curve keys, (key, id)
- * sort, leaf wrapping, summaries) in ONE persistent kernel launch: each thread
- * block takes whole indexes, largest first, from an atomic queue (or, see
- * psi_batch_create, in the launches of one sort of the whole batch).  Each index
- * gets exactly the layout psi_build would give it.  d_pts [total][dim] and
+ * sort, leaf wrapping, summaries): in one persistent kernel launch, whose thread
+ * blocks take whole indexes, largest first, from an atomic queue, or, where
+ * psi_batch_create chose device-wide sorts, in some twenty launches over the
+ * whole batch.  Each index gets exactly the layout psi_build would give it.  d_pts [total][dim] and
  * d_ids [total] are read during the call only. */
 psi_status psi_batch_build(psi_batch *b, const int32_t *d_pts, const uint32_t *d_ids, void *stream);
 
@@ -180,7 +182,7 @@ psi_status psi_batch_knn_reserve(psi_batch *b, int64_t max_queries, void *stream
 
 /* k-NN (Sec 2.2) for queries grouped by index: d_qoffsets (DEVICE, nidx+1
  * entries) gives the queries [qoff[i], qoff[i+1]) that ask index i.  Results as
- * in psi_knn, one launch for all indexes.  nq <= the reserved capacity. */
+ * in psi_knn, in the same launches for all indexes.  nq <= the reserved capacity. */
 psi_status psi_batch_knn(psi_batch *b, const int32_t *d_q, const int64_t *d_qoffsets, int64_t nq, int32_t k,
                          uint32_t *d_ids, int64_t *d_d2, void *stream);
 

@@ -1,4 +1,5 @@
-// batch.cu -- many independent SPaC indexes built in one persistent launch.
+// batch.cu -- many independent SPaC indexes built in one persistent launch, or,
+// where a few large ones hold most of the points, by device-wide sorts (below).
 //
 // Each thread block takes whole indexes from an atomic work queue (largest
 // first, so the long builds start early) and builds each one alone, with the
@@ -13,8 +14,9 @@
 //   T  runs of equal keys are put in id order;
 //   G  leaf wrapping into blocks of 2*phi slots with boxes and counts;
 //   U  the F-ary summary levels, bottom up.
-// All storage is laid out by the host from the index sizes before the launch,
-// so the launch allocates nothing and can be captured in a CUDA graph.
+// All storage, the sorts' scratch included, is laid out by the host from the
+// index sizes before the build, so a build allocates nothing and can be captured
+// in a CUDA graph.
 #include <algorithm>
 #include <numeric>
 #include <type_traits>
@@ -478,7 +480,8 @@ __global__ __launch_bounds__(256) void k_wide_keys(const int32_t *pts, int64_t n
   __shared__ alignas(16) uint8_t htab[kCurveTabBytes];
   curve_table_init<D, CURVE>(htab);
   __syncthreads();
-  const uint64_t mask = (uint64_t(1) << (D * bits)) - 1;  // (a coordinate out of range is reported; its key stays in range)
+  // (a coordinate out of range is reported; its key stays in range)
+  const uint64_t mask = (uint64_t(1) << (D * bits)) - 1;
   bool bad_any = false;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
     int32_t c[D];
@@ -643,7 +646,8 @@ psi_status build_wide(psi_batch *b, const BuildArgs &a, cudaStream_t s) {
   psi_status st;
   SortResult r;
   EncodeSpec none;
-  PSI_LAUNCH_NAMED("k_wide_keys", (k_wide_keys<D, CURVE>), grid(n), 256, 0, s, a.pts, n, a.bits, b->kA, b->vA, a.status);
+  PSI_LAUNCH_NAMED("k_wide_keys", (k_wide_keys<D, CURVE>), grid(n), 256, 0, s, a.pts, n, a.bits, b->kA, b->vA,
+                   a.status);
   if ((st = sort_pairs(none, b->kA, b->vA, n, 8, nullptr, b->kB, b->vB, b->kA, b->vA, a.status, s, &r, 0,
                        b->sort_scratch)))
     return st;
@@ -661,8 +665,9 @@ psi_status build_wide(psi_batch *b, const BuildArgs &a, cudaStream_t s) {
   PSI_LAUNCH(k_wide_ties, grid(n), 256, 0, s, r.keys, r.vals, a.ids, b->d_off, b->nidx, n, longs, b->d_nhard);
   PSI_LAUNCH(k_wide_tie_long, num_sms(), 1024, 0, s, r.keys, r.vals, a.ids, b->d_off, b->nidx, longs, b->d_nhard);
   const int64_t leaves = b->block_off[b->nidx];
-  PSI_LAUNCH_NAMED("k_wide_gather", k_wide_gather<D>, (int)std::min<int64_t>(ceil_div(leaves, 8), (int64_t)num_sms() * 32),
-                   256, 0, s, r.keys, r.vals, a, leaves);
+  PSI_LAUNCH_NAMED("k_wide_gather", k_wide_gather<D>,
+                   (int)std::min<int64_t>(ceil_div(leaves, 8), (int64_t)num_sms() * 32), 256, 0, s, r.keys, r.vals, a,
+                   leaves);
   PSI_LAUNCH_NAMED("k_wide_summary", k_wide_summary<D>, std::min(b->nidx, num_sms() * 4), 512, 0, s, a);
   PSI_CK(cudaGetLastError());
   return PSI_OK;
@@ -1024,8 +1029,8 @@ static psi_status batch_knn(psi_batch *b, const int32_t *d_q, const int64_t *d_q
   hard.q = seed.pos + nq;  // the other half of that buffer, and the sort's free position buffer
   hard.pos = r.vals == b->qv0 ? b->qv1 : b->qv0;
   hard.n = b->d_nhard;
-  return run_knn_roots(tv, b->total, d_q, nq, k, r.vals, b->d_qroot, b->D, d_ids, d_d2, b->d_status, d_stats, s, seed, -1, false,
-                       hard);
+  return run_knn_roots(tv, b->total, d_q, nq, k, r.vals, b->d_qroot, b->D, d_ids, d_d2, b->d_status, d_stats, s, seed,
+                       -1, false, hard);
 }
 
 psi_status psi_batch_knn(psi_batch *b, const int32_t *d_q, const int64_t *d_qoffsets, int64_t nq, int32_t k,

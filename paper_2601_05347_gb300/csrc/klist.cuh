@@ -291,7 +291,8 @@ __device__ __forceinline__ void klist_flush(KList<KPL> &kl, KWait &wt, int &nw, 
 
 // nw: candidates waiting (at most 31 between calls).
 template <int KPL>
-__device__ __forceinline__ void klist_wait(KList<KPL> &kl, KWait &wt, int &nw, bool in, int64_t d2, uint32_t id, int k) {
+__device__ __forceinline__ void klist_wait(KList<KPL> &kl, KWait &wt, int &nw, bool in, int64_t d2, uint32_t id,
+                                           int k) {
   const uint32_t m = __ballot_sync(0xFFFFFFFFu, in);
   if (in) {
     const int p = nw + __popc(m & ((1u << (threadIdx.x & 31)) - 1u));

@@ -751,7 +751,8 @@ __device__ __forceinline__ bool leaf_first(uint64_t lk, uint32_t lid, uint64_t b
   return lk < bk || (lk == bk && lid <= bid);
 }
 
-// New point p (of nc) of a dirty leaf x in segment g.  Insert: found by a merge-path search over the leaf's points and its slice.
+// New point p (of nc) of a dirty leaf x in segment g (insert): found by a
+// merge-path search over the leaf's points and its slice.
 template <int D>
 __device__ __forceinline__ void seg_insert_at(const SegArgs &a, int64_t x, int64_t g, int64_t p) {
   const uint32_t s0 = a.pl.ref[x];

@@ -1,6 +1,8 @@
 // query.cu -- batched k-NN, range count and range list (Sec 2.2) on either
-// tree layout (SPaC summary tree or P-Orth), one warp per query, queries taken
-// in curve order so that neighbouring warps walk the same nodes out of L2.
+// tree layout (SPaC summary tree or P-Orth), one warp per query (k-NN of k <= 32
+// over many queries: two per warp, and of k <= 16 one per thread, knn_lane.cu),
+// queries taken in curve order so that neighbouring warps walk the same nodes
+// out of L2.
 //
 // k-NN: depth-first traversal that enters children in increasing order of
 // their box distance (Appendix "Implementation Details": subtrees are visited
@@ -9,7 +11,7 @@
 // per lane; each level of the current path keeps its children's distance keys
 // and a bitmask of those still to visit in shared memory, and a warp minimum
 // picks the next one.  The search starts from seed leaves at the query's own
-// curve position (SPaC; P-Orth for k > 32).  The k best (d2, id) pairs live in
+// curve position (SPaC, and P-Orth queries that are sorted).  The k best (d2, id) pairs live in
 // a KList (klist.cuh).  Squared distances are exact int64 (|dx| < 2^31 for
 // coordinates in [0, 2^31)).
 //
@@ -1024,12 +1026,12 @@ __device__ __forceinline__ void seg_sort(uint32_t *ids, int len, uint32_t *sm) {
 // segment up to 1024 ids, then blocks of 64, 128 and 512 threads, then
 // k_sort_seg_any.  Many values per thread keep most of the network in registers:
 // at 1024 ids, 15 of its 55 stages are shuffles (whose rate bounds it) with 32
-// values per thread; 28 are between threads with 8.  The classes are listed first and every warp or block takes the next
-// segment of its list: taken in strides over all segments, some find more
-// of their class than others.  5e4 boxes of 1259 ids on
-// average (6.3e7 ids): 590 us, against 6.1 ms for one 1024-thread block per
-// segment with a network in shared memory and a barrier per stage; bound by
-// instruction issue (about 110 per id and 32 lanes).
+// values per thread; 28 are between threads with 8.  The classes are listed
+// first and every warp or block takes the next segment of its list: taken in
+// strides over all segments, some find more of their class than others.  5e4
+// boxes of 1259 ids on average (6.3e7 ids): 590 us, against 6.1 ms for one
+// 1024-thread block per segment with a network in shared memory and a barrier
+// per stage; bound by instruction issue (about 110 per id and 32 lanes).
 constexpr int kSegClasses = 5;
 constexpr int kSeg0 = 1024, kSeg1 = 2048, kSeg2 = 4096, kSeg3 = 16384;  // largest of classes 0 to 3
 
@@ -1183,7 +1185,8 @@ psi_status sort_segments(const int64_t *offsets, int64_t nq, uint32_t *ids, cuda
   PSI_CK(cudaMemsetAsync(ctr.p, 0, sizeof(uint32_t) * 2 * kSegClasses, s));
   const SegLists l{list.p, ctr.p, nq};
   PSI_LAUNCH(k_seg_classes, (int)std::min<int64_t>(ceil_div(nq, 256), (int64_t)num_sms() * 8), 256, 0, s, offsets, l);
-  PSI_LAUNCH(k_sort_seg_warp, (int)std::min<int64_t>(ceil_div(nq, 4), (int64_t)num_sms() * 8), 128, 0, s, offsets, l, ids);
+  PSI_LAUNCH(k_sort_seg_warp, (int)std::min<int64_t>(ceil_div(nq, 4), (int64_t)num_sms() * 8), 128, 0, s, offsets, l,
+             ids);
   if ((st = launch_sort_seg<64, 1>(offsets, l, ids, s)) || (st = launch_sort_seg<128, 2>(offsets, l, ids, s)) ||
       (st = launch_sort_seg<512, 3>(offsets, l, ids, s)) || (st = launch_sort_seg_any<true>(offsets, l, ids, s)))
     return st;
@@ -1267,7 +1270,8 @@ static int64_t lane_min_queries(int sms, int D, int k, bool porth, bool batch, i
 // 6e5 2082 / 3034; 3D uniform 1e8 points 32-NN 2e4 1023 / 256, 6e5 8781 / 5345.
 static int64_t porth_single_max(int D, int k, int64_t n) {
   const double m = (double)n / 1e6;
-  const double line = D == 2 ? 7450 * std::pow((double)k, 0.7) * std::pow(m, 0.3) : 5960 * k * std::pow(std::max(m, 0.6), 0.6);
+  const double line =
+      D == 2 ? 7450 * std::pow((double)k, 0.7) * std::pow(m, 0.3) : 5960 * k * std::pow(std::max(m, 0.6), 0.6);
   return (int64_t)std::max(line, 12000.0);
 }
 static bool porth_single(int D, int k, int64_t nq, int64_t n) { return nq < porth_single_max(D, k, n); }

@@ -155,7 +155,7 @@ __device__ __forceinline__ void sort_leaf_block(Pool &pool, uint32_t s0, int cnt
 }
 
 // Sorts, in place, the block of every leaf that will be re-wrapped.  A warp
-// takes 32 leaves: one lane per leaf finds the few that overflow, then the
+// takes lpw leaves: one lane per leaf finds the few that overflow, then the
 // warp sorts each of those.
 template <int D, int R>
 __global__ void k_sort_overflow_leaves(const int32_t *ncnt, const uint32_t *nref, const int32_t *sbeg,
@@ -248,7 +248,7 @@ __device__ __forceinline__ bool leaf_before_slice(const InsertArgs &a, uint32_t 
   return a.pool.pid[ls] <= a.rid[bi];
 }
 
-// A warp takes 32 new leaf positions: a lane copies the descriptor of an
+// A warp takes lpw new leaf positions: a lane copies the descriptor of an
 // untouched leaf (most of them), then the warp builds each touched one.
 template <int D>
 __global__ void k_insert_apply(InsertArgs a) {
@@ -404,7 +404,7 @@ __global__ void k_insert_apply(InsertArgs a) {
 }
 
 // Insert that splits no leaf: every touched leaf appends its slice in place
-// (its block has room); untouched leaves are not visited.  A warp takes 32
+// (its block has room); untouched leaves are not visited.  A warp takes lpw
 // leaves, one lane per leaf finds those with a slice.
 template <int D>
 __global__ void k_append_inplace(Leaves lv, Pool pool, const int32_t *sbeg, const int32_t *send, int64_t L,
@@ -470,7 +470,7 @@ __global__ void k_batch_records(const uint32_t *bvals, const int32_t *pts, const
   }
 }
 
-// Remove the points named by each leaf's slice: a warp takes 32 leaves, one
+// Remove the points named by each leaf's slice: a warp takes lpw leaves, one
 // lane per leaf finds those with a slice, then the warp compacts them two at a
 // time (both leaves' points and slice entries requested before either is
 // compacted).  R rows of 32 slots cover a leaf's block (R * 32 >= C).
@@ -669,7 +669,7 @@ struct WrapArgs {
   int C, lpw;
 };
 
-// A warp takes 32 new leaf positions: a lane copies the descriptor of a kept
+// A warp takes lpw new leaf positions: a lane copies the descriptor of a kept
 // leaf, then the warp builds each re-wrapped one (part t of its group).
 template <int D>
 __global__ void k_wrap_apply(WrapArgs a) {
@@ -856,9 +856,9 @@ psi_status spac_insert(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
 
   const int64_t base_block = ix->pool_used;
   if ((st = grow_pool(ix, (base_block + NB) * ix->C, base_block * ix->C, s))) return st;
-#define SORT_LEAVES(DD, RR)                                                                                    \
-  PSI_LAUNCH_NAMED("k_sort_overflow_leaves", (k_sort_overflow_leaves<DD, RR>), warp_grid(ceil_div(L, lpw)), 256, 0, s, ix->nodes.cnt, ix->nodes.ref, sbeg.p, \
-                   send.p, L, ix->C, ix->pool, lpw)
+#define SORT_LEAVES(DD, RR)                                                                               \
+  PSI_LAUNCH_NAMED("k_sort_overflow_leaves", (k_sort_overflow_leaves<DD, RR>), warp_grid(ceil_div(L, lpw)), \
+                   256, 0, s, ix->nodes.cnt, ix->nodes.ref, sbeg.p, send.p, L, ix->C, ix->pool, lpw)
   if (ix->D == 2) {
     if (ix->C <= 64) SORT_LEAVES(2, 2);
     else SORT_LEAVES(2, MAXPL);
@@ -1000,9 +1000,9 @@ psi_status spac_delete(psi_index *ix, const int32_t *pts, const uint32_t *ids, i
   const int64_t Lnew = h3[0], NB = h3[1];
   const int64_t base_block = ix->pool_used;
   if ((st = grow_pool(ix, (base_block + NB) * ix->C, base_block * ix->C, s))) return st;
-#define SORT_LEAVES(DD, RR)                                                                                    \
-  PSI_LAUNCH_NAMED("k_sort_flagged_leaves", (k_sort_flagged_leaves<DD, RR>), warp_grid(ceil_div(L, lpw)), 256, 0, s, ix->nodes.cnt, ix->nodes.ref, ingroup.p, \
-                   L, ix->pool, lpw)
+#define SORT_LEAVES(DD, RR)                                                                             \
+  PSI_LAUNCH_NAMED("k_sort_flagged_leaves", (k_sort_flagged_leaves<DD, RR>), warp_grid(ceil_div(L, lpw)), \
+                   256, 0, s, ix->nodes.cnt, ix->nodes.ref, ingroup.p, L, ix->pool, lpw)
   if (ix->D == 2) {
     if (ix->C <= 64) SORT_LEAVES(2, 2);
     else SORT_LEAVES(2, MAXPL);

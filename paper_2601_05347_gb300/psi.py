@@ -282,7 +282,7 @@ class Index:
 
 class Batch:
     """Many independent SPaC indexes over one concatenated point array, built in
-    one persistent launch (psi_batch_*)."""
+    one persistent launch or by device-wide sorts (psi_batch_*, batch_device_wide)."""
 
     def __init__(self, offsets, *, dim: int = 2, kind: int | str = SPAC_H, leaf_size: int = 32,
                  coord_bits: int | None = None, fanout: int = 32, threads: int = 0, radix_bits: int = 0,
