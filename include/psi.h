@@ -264,7 +264,8 @@ psi_status psi_test_sort_withheld_tile(uint64_t *d_keys, uint32_t *d_vals, int64
 
 /* Test hook of the k-NN dispatch: the kernel that psi_knn takes for nq >= 4096
  * queries on one index of n points and a GPU of sms multiprocessors: 'L' one
- * query per thread, 'S' one per warp, 'G' two per warp.  No GPU needed. */
+ * query per thread, 'S' one per warp, 'G' two per warp; 0 for arguments that
+ * psi_knn would not take.  No GPU needed. */
 int32_t psi_test_knn_form(int32_t dim, int32_t k, int32_t porth, int64_t nq, int64_t n, int32_t sms);
 
 /* ---- Instrumentation ---------------------------------------------------- */

@@ -1502,6 +1502,7 @@ psi_status run_range_emit(const psi_index *ix, const int32_t *boxes, int64_t nq,
 // curve order on one index ('L' one query per thread, 'S' one per warp, 'G' two).
 extern "C" int32_t psi_test_knn_form(int32_t dim, int32_t k, int32_t porth, int64_t nq, int64_t n, int32_t sms) {
   using namespace psi;
+  if ((dim != 2 && dim != 3) || k < 1 || k > 128 || sms < 1 || n < 0) return 0;
   if (nq >= lane_min_queries(sms, dim, k, porth != 0, false, n)) return 'L';
   if (k > 32 || (porth && porth_single(dim, k, nq, n))) return 'S';
   return 'G';
