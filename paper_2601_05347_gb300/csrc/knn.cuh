@@ -63,20 +63,25 @@ struct KnnArgs {
 // list is in the order in which warps came to append to it, while neighbours of
 // the curve order read the same nodes: 2e6 8-NN of uniform queries on 3e6 Varden
 // points (2D P-Orth), listed 12.2 ms, in curve order 9.1.
+// (Without a list everything is read from the arguments, which cost no registers.)
+template <bool LIST>
 struct KnnTake {
-  const uint32_t *order, *pos;
-  int64_t nq;
-  __device__ __forceinline__ KnnTake(const KnnArgs &a, bool list) : order(a.order), pos(a.seed.pos), nq(a.nq) {
-    if (!list) return;
-    nq = (int64_t)*a.d_nq;
-    const bool mine = nq >= a.list_lo && nq < a.list_hi;
-    if (4 * nq >= 3 * a.nq) {
-      order = a.all_order;
-      pos = a.all_pos;
-      nq = a.nq;
-    }
-    if (!mine) nq = 0;
+  const KnnArgs &a;
+  const uint32_t *order = nullptr, *seeds = nullptr;
+  int64_t number = 0;
+  __device__ __forceinline__ explicit KnnTake(const KnnArgs &args) : a(args) {
+    if (!LIST) return;
+    const int64_t n = (int64_t)*a.d_nq;
+    const bool all = 4 * n >= 3 * a.nq;
+    order = all ? a.all_order : a.order;
+    seeds = all ? a.all_pos : a.seed.pos;
+    number = n < a.list_lo || n >= a.list_hi ? 0 : all ? a.nq : n;
   }
+  __device__ __forceinline__ int64_t nq() const { return LIST ? number : a.nq; }
+  __device__ __forceinline__ int64_t query(int64_t i) const {
+    return LIST ? (int64_t)order[i] : a.order ? (int64_t)a.order[i] : i;
+  }
+  __device__ __forceinline__ uint32_t pos(int64_t i) const { return LIST ? seeds[i] : a.seed.pos[i]; }
 };
 
 // Per-warp depth-first stack of the k-NN search: an expanded node pushes at

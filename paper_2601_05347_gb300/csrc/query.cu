@@ -199,8 +199,8 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   KWait *wt = &s_wait[KPL > 1 ? w : 0];
   const int64_t warps = (int64_t)gridDim.x * QW;
-  const KnnTake take(a, LIST);
-  const int64_t nq = take.nq;
+  const KnnTake<LIST> take(a);
+  const int64_t nq = take.nq();
   const TreeView &t = a.t;
   __shared__ alignas(16) uint8_t s_tab[SELF ? kCurveTabBytes : 16];
   if (SELF && a.seed.curve == CURVE_HILBERT) {
@@ -209,7 +209,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
   }
   unsigned long long n_int = 0, n_leaf = 0, n_pts = 0, n_kids = 0;
   for (int64_t qi = (int64_t)blockIdx.x * QW + w; qi < nq; qi += warps) {
-    const int64_t q = take.order ? (int64_t)take.order[qi] : qi;
+    const int64_t q = take.query(qi);
     int32_t qc[D];
 #pragma unroll
     for (int d = 0; d < D; ++d) qc[d] = a.q[q * D + d];
@@ -234,7 +234,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn(KnnArgs a, KnnStats stats) {
       s_lo = s_hi = seed_search_warp(sd.sep_key, sd.L, key);
       knn_scan_leaf<D, KPL, true>(t, (uint32_t)s_lo, qc, kl, wt, nw, a.k);
     } else if (sd.qkey && root >= 0) {
-      const int64_t pos = take.pos[qi];  // k_knn_seed
+      const int64_t pos = take.pos(qi);  // k_knn_seed
       if (L > 0) {
         // P-Orth: pos is a position in the key-ordered leaf list
         const int64_t j = sd.leaf_node ? (int64_t)sd.leaf_node[pos] : pos;
@@ -546,8 +546,8 @@ __global__ __launch_bounds__(QW * 32) void k_knn_group(KnnArgs a, KnnStats stats
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const TreeView &t = a.t;
   const KnnSeed &sd = a.seed;
-  const KnnTake take(a, LIST);
-  const int64_t nq = take.nq;
+  const KnnTake<LIST> take(a);
+  const int64_t nq = take.nq();
   const int64_t ngroups = (nq + G - 1) / G;
   unsigned long long n_int = 0, n_leaf = 0, n_pts = 0, n_kids = 0;
   for (int64_t gi = (int64_t)blockIdx.x * QW + w; gi < ngroups; gi += (int64_t)gridDim.x * QW) {
@@ -558,10 +558,10 @@ __global__ __launch_bounds__(QW * 32) void k_knn_group(KnnArgs a, KnnStats stats
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       const int64_t qi = qi0 + min(g, ng - 1);  // a short last group repeats its last query
-      const int64_t q = take.order ? (int64_t)take.order[qi] : qi;
+      const int64_t q = take.query(qi);
 #pragma unroll
       for (int d = 0; d < D; ++d) qc[g][d] = a.q[q * D + d];
-      seed[g] = !sd.qkey ? 0xFFFFFFFFu : sd.leaf_node ? (uint32_t)sd.leaf_node[take.pos[qi]] : take.pos[qi];
+      seed[g] = !sd.qkey ? 0xFFFFFFFFu : sd.leaf_node ? (uint32_t)sd.leaf_node[take.pos(qi)] : take.pos(qi);
     }
     KList<1> kl[G];
 #pragma unroll
@@ -749,7 +749,7 @@ __global__ __launch_bounds__(QW * 32) void k_knn_group(KnnArgs a, KnnStats stats
 #pragma unroll
     for (int g = 0; g < G; ++g) {
       if (g < ng && lane < a.k) {
-        const int64_t q = take.order ? (int64_t)take.order[qi0 + g] : qi0 + g;
+        const int64_t q = take.query(qi0 + g);
         a.out_id[q * a.k + lane] = kl[g].i[0];
         a.out_d2[q * a.k + lane] = kl[g].d[0];
       }
