@@ -925,10 +925,23 @@ __global__ __launch_bounds__(QW * 32) void k_range(RangeArgs a) {
 // Bitonic sort of T * E values held E per thread (value e of thread t at
 // position t * E + e) by a group of T threads: strides below E between a
 // thread's own registers, strides below 32 E by warp shuffles, the others
-// through shared memory ([E][T]; T > 32 only).
-template <int T, int E>
+// through shared memory ([E][T]; T > 32 only).  HALF: the group is one of the
+// halves of a block of 2 T threads, with a barrier of its own.
+template <int T, bool HALF>
+__device__ __forceinline__ void seg_sync() {
+  if (T == 32)
+    __syncwarp();
+  else if (HALF && threadIdx.x < T)  // (numbers known to the compiler: three barriers in all)
+    asm volatile("bar.sync 1, %0;" ::"n"(T) : "memory");
+  else if (HALF)
+    asm volatile("bar.sync 2, %0;" ::"n"(T) : "memory");
+  else
+    __syncthreads();
+}
+
+template <int T, int E, bool HALF = false>
 __device__ __forceinline__ void seg_bitonic(uint32_t (&v)[E], uint32_t *sm) {
-  const int t = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  const int t = T == 32 || HALF ? (int)(threadIdx.x & (T - 1)) : (int)threadIdx.x;
   // strides from .. 1 between the thread's own values: stage k < E, whose runs
   // alternate inside the thread, or (k >= E) an ascending merge
   auto own = [&](int from, int k) {
@@ -967,10 +980,10 @@ __device__ __forceinline__ void seg_bitonic(uint32_t (&v)[E], uint32_t *sm) {
     if (T > 32) {
 #pragma unroll 1
       for (; j >= 32 * E; j >>= 1) {
-        __syncthreads();
+        seg_sync<T, HALF>();
 #pragma unroll
         for (int e = 0; e < E; ++e) sm[e * T + t] = v[e];
-        __syncthreads();
+        seg_sync<T, HALF>();
         const int x = t ^ (j / E);
         const bool low = (t & (j / E)) == 0;
 #pragma unroll
@@ -996,35 +1009,29 @@ __device__ __forceinline__ void seg_bitonic(uint32_t (&v)[E], uint32_t *sm) {
 // Sorts ids[0, len), len <= T * E.  The order of the values on the way in is
 // free, so they are read coalesced; they leave through shared memory, where
 // the group holds T * (E + 1) words.
-template <int T, int E>
+template <int T, int E, bool HALF = false>
 __device__ __forceinline__ void seg_sort(uint32_t *ids, int len, uint32_t *sm) {
-  const int t = T == 32 ? (int)(threadIdx.x & 31) : (int)threadIdx.x;
+  const int t = T == 32 || HALF ? (int)(threadIdx.x & (T - 1)) : (int)threadIdx.x;
   uint32_t v[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) v[e] = e * T + t < len ? ids[e * T + t] : 0xFFFFFFFFu;
-  seg_bitonic<T, E>(v, sm);
-  auto sync = [] {
-    if (T == 32)
-      __syncwarp();
-    else
-      __syncthreads();
-  };
-  sync();
+  seg_bitonic<T, E, HALF>(v, sm);
+  seg_sync<T, HALF>();
   constexpr int S = E > 1 ? E + 1 : 1;  // a word of padding per thread: no bank conflicts
 #pragma unroll
   for (int e = 0; e < E; ++e) sm[t * S + e] = v[e];
-  sync();
+  seg_sync<T, HALF>();
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int p = e * T + t;
     if (p < len) ids[p] = sm[p / E * S + p % E];
   }
-  sync();
+  seg_sync<T, HALF>();
 }
 
 // The segments by length, each class sorted by a kernel of its own: a warp per
-// segment up to 1024 ids, then blocks of 64, 128 and 512 threads, then
-// k_sort_seg_any.  Many values per thread keep most of the network in registers:
+// segment up to 1024 ids, then 64, 128 and 512 threads (the first two in one
+// launch: a launch costs a small report 4 us), then k_sort_seg_any.  Many values per thread keep most of the network in registers:
 // at 1024 ids, 15 of its 55 stages are shuffles (whose rate bounds it) with 32
 // values per thread; 28 are between threads with 8.  The classes are listed
 // first and every warp or block takes the next segment of its list: taken in
@@ -1087,24 +1094,51 @@ __global__ __launch_bounds__(128, 8) void k_sort_seg_warp(const int64_t *offsets
   }
 }
 
-// Class C: a block of T threads per segment, of up to 32 T ids.
-template <int T, int C>
-__global__ __launch_bounds__(T, 1024 / T) void k_sort_seg_block(const int64_t *offsets, SegLists l, uint32_t *ids) {
-  extern __shared__ uint32_t sm_seg[];  // T * 33
-  __shared__ uint32_t next;
-  const uint32_t n = l.ctr[C];
-  for (;;) {
-    if (threadIdx.x == 0) next = atomicAdd(&l.ctr[kSegClasses + C], 1u);
-    __syncthreads();
-    const uint32_t x = next;
-    __syncthreads();
+// The next segment of class c for a group of threads (lead: one of them), or
+// its number past the class's end.
+template <int T, bool HALF>
+__device__ __forceinline__ uint32_t seg_next(const SegLists &l, int c, uint32_t &slot, bool lead) {
+  if (lead) slot = atomicAdd(&l.ctr[kSegClasses + c], 1u);
+  seg_sync<T, HALF>();
+  const uint32_t x = slot;
+  seg_sync<T, HALF>();
+  return x;
+}
+
+// Class 1 by the halves of a block, 64 threads each, then class 2 by whole
+// blocks: one launch for both.
+__global__ __launch_bounds__(128, 8) void k_sort_seg_mid(const int64_t *offsets, SegLists l, uint32_t *ids) {
+  __shared__ uint32_t sm[128 * 33];
+  __shared__ uint32_t next[2];
+  const int h = threadIdx.x >> 6;
+  for (const uint32_t n = l.ctr[1];;) {
+    const uint32_t x = seg_next<64, true>(l, 1, next[h], (threadIdx.x & 63) == 0);
     if (x >= n) break;
-    const int64_t q = l.list[C * l.nq + x], b = offsets[q];
+    const int64_t q = l.list[l.nq + x], b = offsets[q];
+    seg_sort<64, 32, true>(ids + b, (int)(offsets[q + 1] - b), sm + h * (64 * 33));
+  }
+  __syncthreads();
+  for (const uint32_t n = l.ctr[2];;) {
+    const uint32_t x = seg_next<128, false>(l, 2, next[0], threadIdx.x == 0);
+    if (x >= n) break;
+    const int64_t q = l.list[2 * l.nq + x], b = offsets[q];
+    seg_sort<128, 32>(ids + b, (int)(offsets[q + 1] - b), sm);
+  }
+}
+
+// Class 3: a block of 512 threads per segment.
+__global__ __launch_bounds__(512, 2) void k_sort_seg_block(const int64_t *offsets, SegLists l, uint32_t *ids) {
+  extern __shared__ uint32_t sm_seg[];  // 512 * 33
+  __shared__ uint32_t next;
+  for (const uint32_t n = l.ctr[3];;) {
+    const uint32_t x = seg_next<512, false>(l, 3, next, threadIdx.x == 0);
+    if (x >= n) break;
+    const int64_t q = l.list[3 * l.nq + x], b = offsets[q];
     const int len = (int)(offsets[q + 1] - b);
-    if (C == 3 && len <= 16 * T)
-      seg_sort<T, 16>(ids + b, len, sm_seg);
+    if (len <= 16 * 512)
+      seg_sort<512, 16>(ids + b, len, sm_seg);
     else
-      seg_sort<T, 32>(ids + b, len, sm_seg);
+      seg_sort<512, 32>(ids + b, len, sm_seg);
   }
 }
 
@@ -1153,16 +1187,6 @@ __global__ __launch_bounds__(kSegT, 1) void k_sort_seg_any(const int64_t *offset
   }
 }
 
-template <int T, int C>
-psi_status launch_sort_seg(const int64_t *offsets, const SegLists &l, uint32_t *ids, cudaStream_t s) {
-  const size_t smem = sizeof(uint32_t) * T * 33;
-  if (smem > 48 * 1024)
-    PSI_CK(cudaFuncSetAttribute(k_sort_seg_block<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  PSI_LAUNCH_NAMED("k_sort_seg_block", (k_sort_seg_block<T, C>),
-                   (int)std::min<int64_t>(l.nq, (int64_t)num_sms() * (1024 / T)), T, smem, s, offsets, l, ids);
-  return PSI_OK;
-}
-
 template <bool LIST>
 psi_status launch_sort_seg_any(const int64_t *offsets, const SegLists &l, uint32_t *ids, cudaStream_t s) {
   const size_t smem = LIST ? 0 : sizeof(uint32_t) * kSegT * 17;
@@ -1187,10 +1211,11 @@ psi_status sort_segments(const int64_t *offsets, int64_t nq, uint32_t *ids, cuda
   PSI_LAUNCH(k_seg_classes, (int)std::min<int64_t>(ceil_div(nq, 256), (int64_t)num_sms() * 8), 256, 0, s, offsets, l);
   PSI_LAUNCH(k_sort_seg_warp, (int)std::min<int64_t>(ceil_div(nq, 4), (int64_t)num_sms() * 8), 128, 0, s, offsets, l,
              ids);
-  if ((st = launch_sort_seg<64, 1>(offsets, l, ids, s)) || (st = launch_sort_seg<128, 2>(offsets, l, ids, s)) ||
-      (st = launch_sort_seg<512, 3>(offsets, l, ids, s)) || (st = launch_sort_seg_any<true>(offsets, l, ids, s)))
-    return st;
-  return PSI_OK;
+  PSI_LAUNCH(k_sort_seg_mid, (int)std::min<int64_t>(nq, (int64_t)num_sms() * 8), 128, 0, s, offsets, l, ids);
+  const size_t smem = sizeof(uint32_t) * 512 * 33;
+  PSI_CK(cudaFuncSetAttribute(k_sort_seg_block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  PSI_LAUNCH(k_sort_seg_block, (int)std::min<int64_t>(nq, (int64_t)num_sms() * 2), 512, smem, s, offsets, l, ids);
+  return launch_sort_seg_any<true>(offsets, l, ids, s);
 }
 
 // Grid of a grid-stride query kernel: the blocks that are resident at once
